@@ -53,6 +53,7 @@ struct Level {
     double *u = nullptr, *f = nullptr, *c0 = nullptr, *c1 = nullptr, *ur = nullptr;  // FP64
     float *e = nullptr, *r = nullptr, *m = nullptr, *inv = nullptr;                 // FP32
     float *e2 = nullptr;  // finest level: second correction buffer of the fused colour passes
+    float *eb = nullptr;  // levels smoothed in one launch per direction: the black half between the two
 };
 
 // one patch of a chain (gr_patch): ghosted (n + 4)^3 FP64 work arrays
@@ -544,6 +545,24 @@ void vcycle32(gr_ctx *c, int kind32, int nu1, int nu2, Start start, float *uh = 
     // coarse level relaxed by separate launches (above the tail, not the 2^3
     // solve) also gets its first red pass from the restriction
     auto first_red_from_restrict = [&](int lc) { return nu1 > 0 && lc >= 1 && lc > (tail ? tail : 0); };
+    // levels 64^3 .. 2^3 in one cluster launch below a 128^3 or finer top
+    const bool clus = tail && c->cluster_on && top >= 6 && nu1 > 0 && nu2 > 0 && gr::coarse_cluster_ok(kind32);
+    const int low = clus ? 5 : tail;  // the levels up to `low` run inside one launch
+    // levels above it that run in one launch per direction
+    auto one_launch = [&](int l) {
+        return tail && l > low && c->lev[l].eb && !c->lev[l].e2 && gr::level_fused_fits(kind32, c->lev[l].n, nu1, nu2);
+    };
+    // pre-smoothing and restriction of such a level; from_r: from e = 0
+    auto level_down = [&](int l, bool from_r) {
+        Level &A = c->lev[l], &C = c->lev[l - 1];
+        const bool fr = first_red_from_restrict(l - 1);
+        gr::level_down(kind32, A.n, from_r, A.e, A.eb, A.r, A.m, A.inv, A.h2, A.ih2, one_launch(l - 1) ? nullptr : C.e,
+                       C.r, C.inv, fr ? C.h2 : 0.0, c->st);
+    };
+    auto level_up = [&](int l, float *uh_, float *ul_) {
+        Level &A = c->lev[l];
+        gr::level_up(kind32, A.n, A.e, A.eb, A.r, A.inv, c->lev[l - 1].e, A.h2, uh_, ul_, c->st);
+    };
     auto down = [&](int l) {
         Level &A = c->lev[l], &C = c->lev[l - 1];
         if (nu1 > 0) {
@@ -589,7 +608,15 @@ void vcycle32(gr_ctx *c, int kind32, int nu1, int nu2, Start start, float *uh = 
             timed(c, cls(GR_PROF_SWEEP32), [&] { smooth(F, nu); });
         }
     };
-    if (start == START_RED_DONE && nu1 > 0) {
+    const bool ftop = one_launch(top);
+    if (ftop) {
+        // the first red pass: made by the level's launch from e = 0, or here from a given e
+        if (start == START_GIVEN)
+            timed(c, cls(GR_PROF_SWEEP32), [&] {
+                gr::sweep_colour<float>(kind32, F.n, F.e, F.r, F.m, F.inv, F.h2, F.ih2, 0.0, 0, c->st, dir_of(F));
+            });
+        timed(c, cls(GR_PROF_RESTRICT), [&] { level_down(top, start == START_ZERO); });
+    } else if (start == START_RED_DONE && nu1 > 0) {
         if (!fused3(nu1, 1)) {
             timed(c, cls(GR_PROF_SWEEP32), [&] {
                 gr::sweep_colour<float>(kind32, F.n, F.e, F.r, F.m, F.inv, F.h2, F.ih2, 0.0, 1, c->st, dir_of(F));
@@ -600,12 +627,13 @@ void vcycle32(gr_ctx *c, int kind32, int nu1, int nu2, Start start, float *uh = 
         if (start != START_GIVEN) cudaMemsetAsync(F.e, 0, sizeof(float) * (size_t)F.n * F.n * F.n, c->st);
         smooth_fine(nu1);
     }
-    timed(c, cls(GR_PROF_RESTRICT), [&] { down(top); });
-    // levels 64^3 .. 2^3 in one cluster launch below a 128^3 or finer top
-    const bool clus = tail && c->cluster_on && top >= 6 && nu1 > 0 && nu2 > 0 && gr::coarse_cluster_ok(kind32);
-    const int low = clus ? 5 : tail;  // the levels up to `low` run inside one launch
+    if (!ftop) timed(c, cls(GR_PROF_RESTRICT), [&] { down(top); });
     timed(c, GR_PROF_COARSE, [&] {
         for (int l = top - 1; l >= (low ? low + 1 : 1); l--) {
+            if (one_launch(l)) {
+                level_down(l, true);
+                continue;
+            }
             smooth_after_restrict(c->lev[l], l);
             down(l);
         }
@@ -639,10 +667,18 @@ void vcycle32(gr_ctx *c, int kind32, int nu1, int nu2, Start start, float *uh = 
             gr::coarsest<float>(kind32, Z.e, Z.r, Z.m, Z.inv, Z.h2, Z.ih2, 0.0, c->st);
         }
         for (int l = low ? low + 1 : 1; l < top; l++) {
+            if (one_launch(l)) {
+                level_up(l, nullptr, nullptr);
+                continue;
+            }
             up(l);
             smooth(c->lev[l], nu2);
         }
     });
+    if (ftop) {
+        timed(c, cls(GR_PROF_PROLONG), [&] { level_up(top, uh, ul); });
+        return;
+    }
     timed(c, cls(GR_PROF_PROLONG), [&] { up(top); });
     if (!uh) {
         smooth_fine(nu2);
@@ -1401,6 +1437,7 @@ gr_status gr_create(int n, double L, void *stream, gr_ctx **out)
         if (st == GR_OK) st = dalloc(c, &A.r, N);
         if (st == GR_OK) st = dalloc(c, &A.m, N);
         if (st == GR_OK) st = dalloc(c, &A.inv, N);
+        if (st == GR_OK && gr::level_fused_fits(KPOISSON, A.n, 2, 2)) st = dalloc(c, &A.eb, N / 2);
     }
     const size_t N = (size_t)n * n * n;
     if (st == GR_OK && n >= c->s3_min && gr::smooth3_fits(KPOISSON, n)) {

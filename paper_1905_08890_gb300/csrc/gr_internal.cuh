@@ -272,6 +272,21 @@ bool coarse_cluster_ok(int kind);
 void coarse_cluster(int kind, float *const *e, float *const *r, const float *const *m, const float *const *inv,
                     const double *h2, const double *ih2, int nu1, int nu2, cudaStream_t st);
 
+// A level of 32^3 or 64^3 smoothed in one launch per direction
+// (level_fused.cu; linear kinds, nu1 = nu2 = 2).  level_down: the pre-smoothing
+// and the restriction: from_r starts from e = 0 (first red pass from r),
+// otherwise e's red half holds the first red pass; eb receives the black half,
+// rc the coarse right-hand side and ec (may be null) the coarse correction's
+// start as resid_restrict_red writes it (h2c = 0: zeros).  level_up: the
+// black half eb corrected from ec, then the post-smoothing; the result goes to
+// e or, with uh and ul, is added to the double-float unknown.
+bool level_fused_fits(int kind, int n, int nu1, int nu2);
+void level_down(int kind, int n, bool from_r, const float *e, float *eb, const float *r, const float *m,
+                const float *inv, double h2, double ih2, float *ec, float *rc, const float *cinv, double h2c,
+                cudaStream_t st);
+void level_up(int kind, int n, float *e, const float *eb, const float *r, const float *inv, const float *ec, double h2,
+              float *uh, float *ul, cudaStream_t st);
+
 // ---- mixed precision -------------------------------------------------------
 // FP64 residual on the fine level; writes r32 = -eps (split), and for KPSI
 // the Jacobian coefficient m32 = -dN/du > 0 and its inverse diagonal inv32.
