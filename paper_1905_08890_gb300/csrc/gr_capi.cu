@@ -476,31 +476,53 @@ void vcycle64(gr_ctx *c, int kind, double rho, int nu1, int nu2)
             for (int col = 0; col < 2; col++)
                 gr::sweep_colour<double>(kind, A.n, A.u, A.f, A.c0, A.c1, A.h2, A.ih2, rho, col, c->st);
     };
+    // after a black pass of a linear kind only red residuals are restricted,
+    // and before a red one only black cells take the correction
     auto down = [&](int l) {
         Level &A = c->lev[l], &C = c->lev[l - 1];
-        gr::resid_restrict<double>(kind, A.n, A.u, A.f, A.c0, A.c1, A.ih2, rho, C.u, C.f, C.ur, fas, c->st);
+        gr::resid_restrict<double>(kind, A.n, A.u, A.f, A.c0, A.c1, A.ih2, rho, C.u, C.f, C.ur, fas, c->st,
+                                   !fas && nu1 > 0);
         if (fas) gr::fas_rhs(C.n, C.u, C.f, C.c0, C.c1, C.ih2, rho, c->st);
     };
     auto up = [&](int l) {
         Level &A = c->lev[l], &C = c->lev[l - 1];
         if (fas) gr::fas_diff(C.n, C.u, C.ur, c->st);
-        gr::prolong_add<double>(A.n, A.u, C.u, c->st);
+        gr::prolong_add64(A.n, A.u, C.u, !fas && nu2 > 0, c->st);
     };
-    Level &F = c->lev[top];
-    timed(c, GR_PROF_SWEEP64, [&] { smooth(F, nu1); });
-    timed(c, GR_PROF_RESTRICT, [&] { down(top); });
-    timed(c, GR_PROF_COARSE, [&] {
-        for (int l = top - 1; l >= 1; l--) {
+    // levels up to 16^3 run in one launch
+    const int low = (c->tail_on && gr::tail64_ok(kind)) ? std::min(top, 3) : 0;
+    auto coarse = [&] {
+        for (int l = top - 1; l > low; l--) {
             smooth(c->lev[l], nu1);
             down(l);
         }
-        Level &Z = c->lev[0];
-        gr::coarsest<double>(kind, Z.u, Z.f, Z.c0, Z.c1, Z.h2, Z.ih2, rho, c->st);
-        for (int l = 1; l < top; l++) {
+        if (low) {
+            const double *c0[4] = {}, *c1[4] = {};
+            double h2[4] = {}, ih2[4] = {};
+            for (int l = 0; l <= low; l++) {
+                c0[l] = c->lev[l].c0;
+                c1[l] = c->lev[l].c1;
+                h2[l] = c->lev[l].h2;
+                ih2[l] = c->lev[l].ih2;
+            }
+            gr::tail64(kind, low, c->lev[low].u, c->lev[low].f, c0, c1, h2, ih2, rho, nu1, nu2, c->st);
+        } else {
+            Level &Z = c->lev[0];
+            gr::coarsest<double>(kind, Z.u, Z.f, Z.c0, Z.c1, Z.h2, Z.ih2, rho, c->st);
+        }
+        for (int l = low + 1; l < top; l++) {
             up(l);
             smooth(c->lev[l], nu2);
         }
-    });
+    };
+    if (low == top) {  // grids up to 16^3: the whole cycle
+        timed(c, GR_PROF_COARSE, coarse);
+        return;
+    }
+    Level &F = c->lev[top];
+    timed(c, GR_PROF_SWEEP64, [&] { smooth(F, nu1); });
+    timed(c, GR_PROF_RESTRICT, [&] { down(top); });
+    timed(c, GR_PROF_COARSE, coarse);
     timed(c, GR_PROF_PROLONG, [&] { up(top); });
     timed(c, GR_PROF_SWEEP64, [&] { smooth(F, nu2); });
 }

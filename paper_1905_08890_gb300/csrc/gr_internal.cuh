@@ -202,9 +202,11 @@ void sweep_colour(int kind, int n, T *u, const T *f, const T *c0, const T *c1, d
 // Residual eps = L(u) - f of the fine level restricted to the coarse level.
 // Correction form (fas = 0): fc = -R eps, uc = 0.  FAS (fas = 1, KPSI):
 // fc = R eps, uc = urc = R u.  c0 is m for KHELM (the operator), s0 for KPSI.
+// red_only (linear kinds, right after a black relaxation pass): the black
+// children's residuals, zero up to rounding, count as zero.
 template <typename T>
 void resid_restrict(int kind, int nf, const T *u, const T *f, const T *c0, const T *c1, double ih2, double rho, T *uc,
-                    T *fc, T *urc, int fas, cudaStream_t st);
+                    T *fc, T *urc, int fas, cudaStream_t st, bool red_only = false);
 // FP32 correction form of the same (KPOISSON or KHELM with m) right after a
 // black relaxation pass: only the red children's residuals enter the average,
 // the black ones being zero up to rounding.  h2c > 0: the coarse correction
@@ -222,6 +224,8 @@ void fas_diff(int nc, double *uc, const double *urc, cudaStream_t st);
 // Fine u += P(uc), cell-centred trilinear.
 template <typename T>
 void prolong_add(int nf, T *u, const T *uc, cudaStream_t st);
+// FP64, black_only when a red pass of a linear equation follows
+void prolong_add64(int nf, double *u, const double *uc, bool black_only, cudaStream_t st);
 // FP32, black children only (a red relaxation of a linear equation follows)
 void prolong_add_black(int nf, float *u, const float *uc, cudaStream_t st, int rev = 0);
 // FP32 coarse = 8-child average of fine (a right-hand side going down)
@@ -286,6 +290,13 @@ void level_down(int kind, int n, bool from_r, const float *e, float *eb, const f
                 cudaStream_t st);
 void level_up(int kind, int n, float *e, const float *eb, const float *r, const float *inv, const float *ec, double h2,
               float *uh, float *ul, cudaStream_t st);
+
+// Levels 2 << top .. 2^3 (top = 1 .. 3) of an FP64 V-cycle in one 16-CTA
+// cluster launch (fp64_tail.cu): u and f of the top level in, u out; c0, c1, h2
+// and ih2 of levels 2^3 (index 0) .. top.  tail64_ok: the device runs such a cluster.
+bool tail64_ok(int kind);
+void tail64(int kind, int top, double *u, const double *f, const double *const *c0, const double *const *c1,
+            const double *h2, const double *ih2, double rho, int nu1, int nu2, cudaStream_t st);
 
 // ---- mixed precision -------------------------------------------------------
 // FP64 residual on the fine level; writes r32 = -eps (split), and for KPSI

@@ -533,6 +533,66 @@ __global__ void __launch_bounds__(kBlock, 5) k_prolong_black4(int lgf, float *__
     }
 }
 
+// FP64 prolongation, one thread per pair of coarse cells K = 2Q, 2Q + 1 and
+// fine row (i, j): the four coarse rows around the fine row, weights 3 and 1
+// per axis (one fused multiply-add each) and one factor 1/64 at the end.  FP64
+// issue bounds it: 16 (BLACK) or 32 operations for two or four cells, against
+// 168 for sixteen in k_prolong_add, whose one thread per sixteen fine cells
+// also leaves a small grid idle (32^3: 12 us a launch, cold).
+template <int BLACK>
+__global__ void __launch_bounds__(kBlock) k_prolong64(int lgf, double *__restrict__ u, const double *__restrict__ uc)
+{
+    pdl_begin();
+    const int lgc = lgf - 1, mc = (1 << lgc) - 1, hc = lgc - 1, mq = (1 << hc) - 1, mf = (1 << lgf) - 1;
+    const int halfc = 1 << (3 * lgc - 1), halff = 1 << (3 * lgf - 1);
+    const int cnt = 1 << (2 * lgf + hc);
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < cnt; t += gridDim.x * blockDim.x) {
+        const int Q = t & mq, j = (t >> hc) & mf, i = t >> (hc + lgf);
+        const int Qm = (Q - 1) & mq, Qp = (Q + 1) & mq;
+        const int I[2] = {i >> 1, ((i >> 1) + ((i & 1) ? 1 : -1)) & mc};
+        const int J[2] = {j >> 1, ((j >> 1) + ((j & 1) ? 1 : -1)) & mc};
+        const int p = (i + j) & 1;  // fine cell k = 4Q + m has colour (p + m) & 1
+        double v[4];
+#pragma unroll
+        for (int a = 0; a < 2; a++) {
+            double y[4];
+#pragma unroll
+            for (int b = 0; b < 2; b++) {
+                const int base = ((I[a] << lgc) + J[b]) << hc;
+                const int ce = ((I[a] + J[b]) & 1) ? halfc : 0, co = halfc - ce;  // even, odd coarse k
+                const double c0 = uc[ce + base + Q], c1 = uc[co + base + Q];
+                double z[4];
+                if (BLACK) {  // the two black children only: m = 1, 3 (p = 0) or m = 0, 2
+                    const double x = p ? uc[co + base + Qm] : uc[ce + base + Qp];
+                    z[0] = p ? fma(3.0, c0, x) : fma(3.0, c0, c1);
+                    z[1] = p ? fma(3.0, c1, c0) : fma(3.0, c1, x);
+                } else {
+                    z[0] = fma(3.0, c0, uc[co + base + Qm]);
+                    z[1] = fma(3.0, c0, c1);
+                    z[2] = fma(3.0, c1, c0);
+                    z[3] = fma(3.0, c1, uc[ce + base + Qp]);
+                }
+#pragma unroll
+                for (int m = 0; m < (BLACK ? 2 : 4); m++) y[m] = b ? y[m] + z[m] : 3.0 * z[m];
+            }
+#pragma unroll
+            for (int m = 0; m < (BLACK ? 2 : 4); m++) v[m] = a ? v[m] + y[m] : 3.0 * y[m];
+        }
+        const int row = (((i << lgf) + j) << (lgf - 1)) + 2 * Q;
+        double2 *blk = reinterpret_cast<double2 *>(u + halff + row);
+        double2 b2 = *blk;
+        b2.x = fma(1.0 / 64.0, BLACK ? v[0] : (p ? v[0] : v[1]), b2.x);
+        b2.y = fma(1.0 / 64.0, BLACK ? v[1] : (p ? v[2] : v[3]), b2.y);
+        *blk = b2;
+        if (!BLACK) {
+            double2 *red = reinterpret_cast<double2 *>(u + row);
+            double2 r2 = *red;
+            r2.x = fma(1.0 / 64.0, p ? v[1] : v[0], r2.x);
+            r2.y = fma(1.0 / 64.0, p ? v[3] : v[2], r2.y);
+            *red = r2;
+        }
+    }
+}
 
 // ---------------------------------------------------------------- 2^3 level
 // Linear kinds: the exact solve (coarsest_exact).  KPSI: Newton red-black
@@ -801,11 +861,15 @@ void sweep_colour(int kind, int n, T *u, const T *f, const T *c0, const T *c1, d
 
 template <typename T>
 void resid_restrict(int kind, int nf, const T *u, const T *f, const T *c0, const T *c1, double ih2, double rho, T *uc,
-                    T *fc, T *urc, int fas, cudaStream_t st)
+                    T *fc, T *urc, int fas, cudaStream_t st, bool red_only)
 {
     const int lgf = log2i(nf);
     const int g = grid_for((int64_t)nf * nf * nf / 8);
-    if (kind == KPOISSON)
+    if (red_only && kind == KPOISSON)
+        GR_LAUNCH((k_resid_restrict<T, KPOISSON, 0, 1>), g, kBlock, st, lgf, u, f, c0, c1, (T)ih2, (T)rho, uc, fc, urc, nullptr, T(0), 0);
+    else if (red_only && kind == KHELM)
+        GR_LAUNCH((k_resid_restrict<T, KHELM, 0, 1>), g, kBlock, st, lgf, u, f, c0, c1, (T)ih2, (T)rho, uc, fc, urc, nullptr, T(0), 0);
+    else if (kind == KPOISSON)
         GR_LAUNCH((k_resid_restrict<T, KPOISSON, 0>), g, kBlock, st, lgf, u, f, c0, c1, (T)ih2, (T)rho, uc, fc, urc, nullptr, T(0), 0);
     else if (kind == KHELM)
         GR_LAUNCH((k_resid_restrict<T, KHELM, 0>), g, kBlock, st, lgf, u, f, c0, c1, (T)ih2, (T)rho, uc, fc, urc, nullptr, T(0), 0);
@@ -882,6 +946,15 @@ void prolong_add(int nf, T *u, const T *uc, cudaStream_t st)
 {
     GR_LAUNCH((k_prolong_add<T>), wave_grid(k_prolong_add<T>, (int64_t)nf * nf * nf / 16), kBlock, st, log2i(nf), u,
               uc, 0);
+}
+
+void prolong_add64(int nf, double *u, const double *uc, bool black_only, cudaStream_t st)
+{
+    const int64_t threads = (int64_t)nf * nf * nf / 4;
+    if (black_only)
+        GR_LAUNCH(k_prolong64<1>, wave_grid(k_prolong64<1>, threads), kBlock, st, log2i(nf), u, uc);
+    else
+        GR_LAUNCH(k_prolong64<0>, wave_grid(k_prolong64<0>, threads), kBlock, st, log2i(nf), u, uc);
 }
 
 template <typename T>
@@ -972,7 +1045,7 @@ void to_float(int64_t cnt, const double *a, float *b, cudaStream_t st)
     template void sweep_colour<T>(int, int, T *, const T *, const T *, const T *, double, double, double, int,     \
                                   cudaStream_t, int);                                                              \
     template void resid_restrict<T>(int, int, const T *, const T *, const T *, const T *, double, double, T *, T *, \
-                                    T *, int, cudaStream_t);                                                       \
+                                    T *, int, cudaStream_t, bool);                                                 \
     template void prolong_add<T>(int, T *, const T *, cudaStream_t);                                               \
     template void coarsest<T>(int, T *, T *, const T *, const T *, double, double, double, cudaStream_t);           \
     template void restrict_coef<T>(int, int, const T *, const T *, T *, T *, double, cudaStream_t);                \
