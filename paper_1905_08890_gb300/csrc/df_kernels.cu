@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kBlock, (resid_min_blocks<KIND, W>()))
                const float *__restrict__ fl, const float *__restrict__ ah, const float *__restrict__ al,
                const float *__restrict__ bh, const float *__restrict__ bl, df cpr, float c5, float ih2,
                float ih2_ref, float *__restrict__ r32, float *__restrict__ m32, float *__restrict__ inv32,
-               const float *__restrict__ inv_in, float *__restrict__ e32, double *__restrict__ partials, int rev,
+               const float *__restrict__ inv_in, float *__restrict__ e32, const Sums sums, int rev,
                const double *__restrict__ fshift, double fsh_scale)
 {
     pdl_begin();
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kBlock, (resid_min_blocks<KIND, W>()))
             }
         }
     }
-    block_sum2f(acc, 0.0f, partials);
+    block_sum2f(acc, 0.0f, sums);
 }
 
 
@@ -243,9 +243,9 @@ __global__ void __launch_bounds__(kBlock)
 
 }  // namespace
 
-int df_resid(int kind, int n, const float *uh, const float *ul, const float *fh, const float *fl, const float *ah,
+void df_resid(int kind, int n, const float *uh, const float *ul, const float *fh, const float *fl, const float *ah,
              const float *al, const float *bh, const float *bl, double h2, double rho, double ref, float *r32,
-             float *m32, float *inv32, const float *inv_in, float *e32, double *partials, cudaStream_t st, int rev,
+             float *m32, float *inv32, const float *inv_in, float *e32, const Sums &sums, cudaStream_t st, int rev,
              const double *fshift)
 {
     const int lgn = log2i(n);
@@ -258,7 +258,7 @@ int df_resid(int kind, int n, const float *uh, const float *ul, const float *fh,
     do {                                                                                                         \
         g = wave_grid(k_df_resid<K, W, S>, threads);                                                             \
         GR_LAUNCH((k_df_resid<K, W, S>), g, kBlock, st, lgn, uh, ul, fh, fl, ah, al, bh, bl, cpr, c5, ih2,       \
-                  ih2_ref, r32, m32, inv32, inv_in, e32, partials, rev, fshift, h2);                             \
+                  ih2_ref, r32, m32, inv32, inv_in, e32, sums, rev, fshift, h2);                             \
     } while (0)
     if (kind == KPOISSON && fshift) {
         if (w == 4) GR_DF_RESID(KPOISSON, 4, true);
@@ -274,7 +274,6 @@ int df_resid(int kind, int n, const float *uh, const float *ul, const float *fh,
         else GR_DF_RESID(KPSI, 2, false);
     }
 #undef GR_DF_RESID
-    return g;
 }
 
 void df_black_update(int kind, int n, const float *e, const float *r, const float *inv, double h2, float *uh,

@@ -130,9 +130,9 @@ struct Acc {
         s.lo = __fadd_rn(s.lo, __fadd_rn(t.lo, x.lo));
         q = __fmaf_rn(x.hi, x.hi, q);
     }
-    // block partials: the warp sums in double-float (FP32) arithmetic, the
-    // eight warp totals in FP64
-    __device__ __forceinline__ void flush(double *partials) const
+    // the warp sums in double-float (FP32) arithmetic, the eight warp totals
+    // and the blocks' in FP64
+    __device__ __forceinline__ void flush(const Sums &sums) const
     {
         __shared__ double sa[kBlock / 32], sb[kBlock / 32];
         df a = s;
@@ -154,32 +154,33 @@ struct Acc {
                 ta += sa[k];
                 tb += sb[k];
             }
-            partials[2 * blockIdx.x] = ta;
-            partials[2 * blockIdx.x + 1] = tb;
+            sums.partials[2 * blockIdx.x] = ta;
+            sums.partials[2 * blockIdx.x + 1] = tb;
         }
+        last_block_sum(sums);
     }
 };
 
 __device__ __forceinline__ df df_scale2(df a, float p2) { return {a.hi * p2, a.lo * p2}; }  // exact for p2 = 2^k
 
 // ---------------------------------------------------------------- sums
-__global__ void __launch_bounds__(kBlock) k_dfs_sum(int64_t cnt, const double *__restrict__ a, double *partials)
+__global__ void __launch_bounds__(kBlock) k_dfs_sum(int64_t cnt, const double *__restrict__ a, const Sums sums)
 {
     pdl_begin();
     Acc acc;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x)
         acc.add(ld(a, t));
-    acc.flush(partials);
+    acc.flush(sums);
 }
 
 __global__ void __launch_bounds__(kBlock)
-    k_dfs_pair_sum(int64_t cnt, const float *__restrict__ h, const float *__restrict__ l, double *partials)
+    k_dfs_pair_sum(int64_t cnt, const float *__restrict__ h, const float *__restrict__ l, const Sums sums)
 {
     pdl_begin();
     Acc acc;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x)
         acc.add(ldp(h, l, t));
-    acc.flush(partials);
+    acc.flush(sums);
 }
 
 // Row reads of four consecutive cells k0 .. k0 + 3 (k0 a multiple of 4) of
@@ -229,7 +230,7 @@ struct PoissonArgs {
 };
 
 template <int SRC>
-__global__ void __launch_bounds__(kBlock, SRC == SRC_SHIFT ? 2 : 3) k_dfs_poisson(int lgn, PoissonArgs a, double *partials)
+__global__ void __launch_bounds__(kBlock, SRC == SRC_SHIFT ? 2 : 3) k_dfs_poisson(int lgn, PoissonArgs a, const Sums sums)
 {
     pdl_begin();
     const int mn = (1 << lgn) - 1;
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(kBlock, SRC == SRC_SHIFT ? 2 : 3) k_dfs_poisso
         stp4(a.fh, a.fl, p, fv);
         stp4(a.uh, a.ul, p, uv);
     }
-    acc.flush(partials);
+    acc.flush(sums);
 }
 
 // ---------------------------------------------------------------- A_ij
@@ -471,7 +472,7 @@ __global__ void __launch_bounds__(kBlock)
     k_dfs_psi(int lgn, df a_scale, df b_scale, const double *__restrict__ psi, const double *__restrict__ s0,
               const float *__restrict__ AAh, const float *__restrict__ AAl, float *__restrict__ uh,
               float *__restrict__ ul, float *__restrict__ ah, float *__restrict__ al, float *__restrict__ bh,
-              float *__restrict__ bl, float *__restrict__ fh, float *__restrict__ fl, double *partials)
+              float *__restrict__ bl, float *__restrict__ fh, float *__restrict__ fl, const Sums sums)
 {
     pdl_begin();
     const int64_t N = (int64_t)1 << (3 * lgn);
@@ -499,7 +500,7 @@ __global__ void __launch_bounds__(kBlock)
         stp4(bh, bl, p, bo);
         stp4(fh, fl, p, zo);
     }
-    acc.flush(partials);
+    acc.flush(sums);
 }
 
 // lapse equation for phi = alpha psi (Eq. sol-scheme-CMC with s = psi^-4 sigma),
@@ -512,7 +513,7 @@ __global__ void __launch_bounds__(kBlock)
                const double *__restrict__ s0, const double *__restrict__ sig, const float *__restrict__ AAh,
                const float *__restrict__ AAl, df two_pi, df k2c, df kdot, float *__restrict__ uh,
                float *__restrict__ ul, float *__restrict__ ah, float *__restrict__ al, float *__restrict__ fh,
-               float *__restrict__ fl, float *__restrict__ m32, float *__restrict__ inv32, double *partials)
+               float *__restrict__ fl, float *__restrict__ m32, float *__restrict__ inv32, const Sums sums)
 {
     pdl_begin();
     const int64_t N = (int64_t)1 << (3 * lgn);
@@ -553,7 +554,7 @@ __global__ void __launch_bounds__(kBlock)
         stf4(m32, p, mo);
         stf4(inv32, p, io);
     }
-    acc.flush(partials);
+    acc.flush(sums);
 }
 
 // shift weight alpha psi^-6 = (alpha psi) psi^-7, natural pairs
@@ -600,22 +601,20 @@ __global__ void __launch_bounds__(kBlock)
 }  // namespace
 
 // ================================================================ launchers
-int dfs_sum(int64_t cnt, const double *a, double *partials, cudaStream_t st)
+void dfs_sum(int64_t cnt, const double *a, const Sums &sums, cudaStream_t st)
 {
-    const int g = grid_for(cnt);
-    GR_LAUNCH(k_dfs_sum, g, kBlock, st, cnt, a, partials);
-    return g;
+    const int g = wave_grid(k_dfs_sum, cnt);
+    GR_LAUNCH(k_dfs_sum, g, kBlock, st, cnt, a, sums);
 }
 
-int dfs_pair_sum(int64_t cnt, const float *h, const float *l, double *partials, cudaStream_t st)
+void dfs_pair_sum(int64_t cnt, const float *h, const float *l, const Sums &sums, cudaStream_t st)
 {
-    const int g = grid_for(cnt);
-    GR_LAUNCH(k_dfs_pair_sum, g, kBlock, st, cnt, h, l, partials);
-    return g;
+    const int g = wave_grid(k_dfs_pair_sum, cnt);
+    GR_LAUNCH(k_dfs_pair_sum, g, kBlock, st, cnt, h, l, sums);
 }
 
-int dfs_mean_rhs(int n, const double *s, const double *sum, double scale, const double *fld, float *uh, float *ul,
-                 float *fh, float *fl, double *partials, cudaStream_t st)
+void dfs_mean_rhs(int n, const double *s, const double *sum, double scale, const double *fld, float *uh, float *ul,
+                 float *fh, float *fl, const Sums &sums, cudaStream_t st)
 {
     const int lgn = log2i(n);
     PoissonArgs a = {};
@@ -629,12 +628,11 @@ int dfs_mean_rhs(int n, const double *s, const double *sum, double scale, const 
     a.fh = fh;
     a.fl = fl;
     const int g = wave_grid(k_dfs_poisson<SRC_MEAN>, (int64_t)n * n * n / (2 * kChunk));
-    GR_LAUNCH(k_dfs_poisson<SRC_MEAN>, g, kBlock, st, lgn, a, partials);
-    return g;
+    GR_LAUNCH(k_dfs_poisson<SRC_MEAN>, g, kBlock, st, lgn, a, sums);
 }
 
-int dfs_div_rhs(int n, double scale, const double *Fx, const double *Fy, const double *Fz, const double *fld,
-                float *uh, float *ul, float *fh, float *fl, double *partials, cudaStream_t st)
+void dfs_div_rhs(int n, double scale, const double *Fx, const double *Fy, const double *Fz, const double *fld,
+                float *uh, float *ul, float *fh, float *fl, const Sums &sums, cudaStream_t st)
 {
     const int lgn = log2i(n);
     PoissonArgs a = {};
@@ -648,12 +646,11 @@ int dfs_div_rhs(int n, double scale, const double *Fx, const double *Fy, const d
     a.fh = fh;
     a.fl = fl;
     const int g = wave_grid(k_dfs_poisson<SRC_DIV>, (int64_t)n * n * n / (2 * kChunk));
-    GR_LAUNCH(k_dfs_poisson<SRC_DIV>, g, kBlock, st, lgn, a, partials);
-    return g;
+    GR_LAUNCH(k_dfs_poisson<SRC_DIV>, g, kBlock, st, lgn, a, sums);
 }
 
-int dfs_shift_rhs(int n, double scale, const float *A, const float *wh, const float *wl, int comp, const double *fld,
-                  float *uh, float *ul, float *fh, float *fl, double *partials, cudaStream_t st)
+void dfs_shift_rhs(int n, double scale, const float *A, const float *wh, const float *wl, int comp, const double *fld,
+                  float *uh, float *ul, float *fh, float *fl, const Sums &sums, cudaStream_t st)
 {
     const int lgn = log2i(n);
     PoissonArgs a = {};
@@ -668,8 +665,7 @@ int dfs_shift_rhs(int n, double scale, const float *A, const float *wh, const fl
     a.fh = fh;
     a.fl = fl;
     const int g = wave_grid(k_dfs_poisson<SRC_SHIFT>, (int64_t)n * n * n / (2 * kChunk));
-    GR_LAUNCH(k_dfs_poisson<SRC_SHIFT>, g, kBlock, st, lgn, a, partials);
-    return g;
+    GR_LAUNCH(k_dfs_poisson<SRC_SHIFT>, g, kBlock, st, lgn, a, sums);
 }
 
 void dfs_aij(int n, double inv2h, double ih2, const double *Vx, const double *Vy, const double *Vz, const double *U,
@@ -683,27 +679,25 @@ void dfs_aij(int n, double inv2h, double ih2, const double *Vx, const double *Vy
               scratch[0], scratch[1], scratch[2], scratch[3], A, AAh, AAl);
 }
 
-int dfs_psi(int n, double h2, const double *psi, const double *s0, const float *AAh, const float *AAl, float *uh,
-            float *ul, float *ah, float *al, float *bh, float *bl, float *fh, float *fl, double *partials,
+void dfs_psi(int n, double h2, const double *psi, const double *s0, const float *AAh, const float *AAl, float *uh,
+            float *ul, float *ah, float *al, float *bh, float *bl, float *fh, float *fl, const Sums &sums,
             cudaStream_t st)
 {
     const int lgn = log2i(n);
     const int g = wave_grid(k_dfs_psi, (int64_t)n * n * n / (2 * kChunk));
     GR_LAUNCH(k_dfs_psi, g, kBlock, st, lgn, df_from_double_host(2.0 * kPi * h2), df_from_double_host(0.125 * h2),
-              psi, s0, AAh, AAl, uh, ul, ah, al, bh, bl, fh, fl, partials);
-    return g;
+              psi, s0, AAh, AAl, uh, ul, ah, al, bh, bl, fh, fl, sums);
 }
 
-int dfs_apsi(int n, double h2, const double *psi, const double *apsi, const double *s0, const double *sig,
+void dfs_apsi(int n, double h2, const double *psi, const double *apsi, const double *s0, const double *sig,
              const float *AAh, const float *AAl, double K2, double Kdot, float *uh, float *ul, float *ah, float *al,
-             float *fh, float *fl, float *m32, float *inv32, double *partials, cudaStream_t st)
+             float *fh, float *fl, float *m32, float *inv32, const Sums &sums, cudaStream_t st)
 {
     const int lgn = log2i(n);
     const int g = wave_grid(k_dfs_apsi, (int64_t)n * n * n / (2 * kChunk));
     GR_LAUNCH(k_dfs_apsi, g, kBlock, st, lgn, (float)h2, df_from_double_host(h2), psi, apsi, s0, sig, AAh, AAl,
               df_from_double_host(2.0 * kPi), df_from_double_host(5.0 / 12.0 * K2), df_from_double_host(Kdot), uh,
-              ul, ah, al, fh, fl, m32, inv32, partials);
-    return g;
+              ul, ah, al, fh, fl, m32, inv32, sums);
 }
 
 void dfs_weight(int n, const double *psi, const double *apsi, float *wh, float *wl, cudaStream_t st)

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kBlock)
 }
 
 // ---------------------------------------------------------------- reductions
-__global__ void __launch_bounds__(kBlock) k_sum_sq(int64_t cnt, const double *__restrict__ a, double *__restrict__ part)
+__global__ void __launch_bounds__(kBlock) k_sum_sq(int64_t cnt, const double *__restrict__ a, const Sums sums)
 {
     pdl_begin();
     double s = 0.0, s2 = 0.0;
@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(kBlock) k_sum_sq(int64_t cnt, const double *__
         s += v;
         s2 += v * v;
     }
-    block_sum2(s, s2, part);
+    block_sum2(s, s2, sums);
 }
 
 __global__ void k_scale_sub_mean(int64_t cnt, double *__restrict__ a, const double *__restrict__ sum, double inv_cnt,
@@ -319,12 +319,10 @@ void deposit(int n, double L, int64_t np, const double *x, const double *u, doub
     deposit_add(n, L, np, x, u, mass, s0, sx, sy, sz, sig, st);
 }
 
-int sum_sq(int64_t cnt, const double *a, double *partials, cudaStream_t st)
+void sum_sq(int64_t cnt, const double *a, const Sums &sums, cudaStream_t st)
 {
-    int g = grid_for(cnt);
-    if (g > kMaxRedBlocks) g = kMaxRedBlocks;
-    GR_LAUNCH(k_sum_sq, g, kBlock, st, cnt, a, partials);
-    return g;
+    const int g = wave_grid(k_sum_sq, cnt);
+    GR_LAUNCH(k_sum_sq, g, kBlock, st, cnt, a, sums);
 }
 
 void scale_sub_mean(int64_t cnt, double *a, const double *sum, double inv_cnt, double scale, cudaStream_t st)

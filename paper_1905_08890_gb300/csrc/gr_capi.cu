@@ -92,6 +92,8 @@ struct gr_ctx {
     double *A6 = nullptr, *AA = nullptr, *tmp = nullptr;
     float *dfu = nullptr, *dff = nullptr, *dfa = nullptr, *dfb = nullptr;  // finest level hi|lo pairs
     double *partials = nullptr, *dscal = nullptr;
+    unsigned *ticket = nullptr;  // of the reductions' last blocks
+    double seq = 0.0;            // number of the last reduction that stores to the host
     double *hscal = nullptr, *hscal_dev = nullptr;  // mapped pinned host scalars and their device alias
     double rho_dep = NAN;
     // what A6/AA hold for the V, U in the fields, and tmp (alpha psi psi^-7) for
@@ -213,11 +215,26 @@ double *field_ptr(const gr_fields *f, int eq)
     }
 }
 
-// device sums (sum, sum of squares) of cnt doubles into c->dscal[0..1]
-void dsum(gr_ctx *c, int64_t cnt, const double *a)
+// where a reduction leaves its sums: out (device); host: also for the next
+// read_scalars
+gr::Sums sums_to(gr_ctx *c, double *out, bool host = false)
 {
-    int g = gr::sum_sq(cnt, a, c->partials, c->st);
-    gr::finalize(c->partials, g, c->dscal, c->st);
+    gr::Sums s;
+    s.partials = c->partials;
+    s.out = out;
+    s.ticket = c->ticket;
+    if (host) {  // two slots in turn: one reduction may be unread while the next is queued
+        s.seq = c->seq += 1.0;
+        s.mapped = c->hscal_dev + 4 * ((long long)s.seq & 1);
+        s.flag = s.mapped + 2;
+    }
+    return s;
+}
+
+// device sums (sum, sum of squares) of cnt doubles into c->dscal[0..1]
+void dsum(gr_ctx *c, int64_t cnt, const double *a, bool host = false)
+{
+    gr::sum_sq(cnt, a, sums_to(c, c->dscal, host), c->st);
 }
 
 cudaEvent_t pool_event(gr_ctx *c)
@@ -263,17 +280,36 @@ void prof_collect(gr_ctx *c)
     cudaGetLastError();
 }
 
-gr_status read_scalars(gr_ctx *c, double *a, double *b)
+// The sums of the last reduction queued with sums_to(..., host), or of the one
+// `back` before it (0 or 1).  Its last block stores them to mapped host memory and then its number: the host polls
+// that instead of synchronising the stream, whose return costs 8 us of idle GPU
+// per cycle.  (Not a copy either: a device-to-host copy would wait for the
+// field copies that host_out keeps in flight on the copy stream.)
+gr_status read_scalars(gr_ctx *c, double *a, double *b, int back = 0)
 {
-    // a kernel store, not a copy: a device-to-host copy would wait for the
-    // field copies that host_out keeps in flight on the copy stream
-    gr::scalars_out(c->dscal, c->hscal_dev, 2, c->st);
-    cudaError_t e = cudaStreamSynchronize(c->st);
-    if (e != cudaSuccess) return fail(GR_ERR_CUDA, "stream: %s", cudaGetErrorString(e));
+    const double seq = c->seq - back;
+    const double *h = c->hscal + 4 * ((long long)seq & 1);
+    auto arrived = [&] {
+        double v;
+        __atomic_load(h + 2, &v, __ATOMIC_ACQUIRE);
+        return v == seq;
+    };
+    for (unsigned spin = 1; !arrived(); spin++) {
+        if (spin & 0xfffu) continue;
+        const cudaError_t e = cudaStreamQuery(c->st);  // an error, or done without a store
+        if (e == cudaErrorNotReady) continue;
+        if (e != cudaSuccess) return fail(GR_ERR_CUDA, "stream: %s", cudaGetErrorString(e));
+        if (arrived()) break;
+        const gr_status s = cuda_check("kernel");
+        return s != GR_OK ? s : fail(GR_ERR_CUDA, "a reduction did not run");
+    }
     gr_status s = cuda_check("kernel");
     if (s != GR_OK) return s;
-    if (c->prof_on) prof_collect(c);
-    const volatile double *h = c->hscal;
+    if (c->prof_on) {
+        const cudaError_t e = cudaStreamSynchronize(c->st);
+        if (e != cudaSuccess) return fail(GR_ERR_CUDA, "stream: %s", cudaGetErrorString(e));
+        prof_collect(c);
+    }
     *a = h[0];
     if (b) *b = h[1];
     return GR_OK;
@@ -286,7 +322,7 @@ gr_status poisson_rhs_finish(gr_ctx *c, Level &F, double *ref)
     const int64_t N = (int64_t)c->n * c->n * c->n;
     dsum(c, N, F.f);
     gr::scale_sub_mean(N, F.f, c->dscal, 1.0 / N, 1.0, c->st);
-    dsum(c, N, F.f);
+    dsum(c, N, F.f, true);
     double s, q;
     gr_status st = read_scalars(c, &s, &q);
     if (st != GR_OK) return st;
@@ -329,7 +365,7 @@ gr_status setup_eq(gr_ctx *c, int eq, const gr_sources *s, const gr_fields *fl, 
     } else if (eq == GR_PSI) {
         ensure_aij(c, fl);
         gr::psi_setup(n, fl->psi, s->s0, c->AA, F.u, F.c0, F.c1, F.f, c->st);
-        dsum(c, N, s->s0);
+        dsum(c, N, s->s0, true);
         double a, q;
         st = read_scalars(c, &a, &q);
         info->ref = 2.0 * kPi * std::sqrt(q / N);
@@ -338,7 +374,7 @@ gr_status setup_eq(gr_ctx *c, int eq, const gr_sources *s, const gr_fields *fl, 
         gr::apsi_setup(n, c->h * c->h, fl->psi, fl->apsi, s->s0, s->sigma, c->AA, K2, Kdot, F.u, F.c0, F.c1, F.f,
                        c->tmp, c->st);
         c->w_fmt = 0;  // tmp now holds psi^5 Kdot
-        dsum(c, N, c->tmp);
+        dsum(c, N, c->tmp, true);
         double a, q;
         st = read_scalars(c, &a, &q);
         info->ref = std::sqrt(q / N);
@@ -386,34 +422,32 @@ gr_status setup_eq_df(gr_ctx *c, int eq, const gr_sources *s, const gr_fields *f
                     c->st);
         c->a_fmt = 2;
     };
-    int g;
     if (eq <= GR_VZ) {
         // lap V_i = 8 pi (s_i - <s_i>)  (Eq. MG-linear-1a; mean removal of Sec. 4.3.1)
-        g = gr::dfs_sum(N, s->s[eq], c->partials, c->st);
-        gr::finalize(c->partials, g, c->dscal, c->st);
-        g = gr::dfs_mean_rhs(n, s->s[eq], c->dscal, 8.0 * kPi * F.h2, fld, uh, ul, fh, fl_, c->partials, c->st);
+        gr::dfs_sum(N, s->s[eq], sums_to(c, c->dscal + 4), c->st);
+        gr::dfs_mean_rhs(n, s->s[eq], c->dscal + 4, 8.0 * kPi * F.h2, fld, uh, ul, fh, fl_, sums_to(c, c->dscal, true),
+                         c->st);
     } else if (eq == GR_U || eq == GR_B_SCALAR) {
         // lap U = -1/4 div V ; lap b = -1/4 div B  (Eqs. MG-linear-1, MG-linear-2)
         double *const *Fv = eq == GR_U ? fl->V : fl->B;
-        g = gr::dfs_div_rhs(n, -0.25 * (0.5 / c->h) * F.h2, Fv[0], Fv[1], Fv[2], fld, uh, ul, fh, fl_, c->partials,
-                            c->st);
+        gr::dfs_div_rhs(n, -0.25 * (0.5 / c->h) * F.h2, Fv[0], Fv[1], Fv[2], fld, uh, ul, fh, fl_,
+                        sums_to(c, c->dscal, true), c->st);
     } else if (eq == GR_PSI) {
         aij();
-        g = gr::dfs_psi(n, F.h2, fl->psi, s->s0, AAh, AAl, uh, ul, c->dfa, c->dfa + N, c->dfb, c->dfb + N, fh, fl_,
-                        c->partials, c->st);
+        gr::dfs_psi(n, F.h2, fl->psi, s->s0, AAh, AAl, uh, ul, c->dfa, c->dfa + N, c->dfb, c->dfb + N, fh, fl_,
+                    sums_to(c, c->dscal, true), c->st);
     } else if (eq == GR_APSI) {
         aij();
-        g = gr::dfs_apsi(n, F.h2, fl->psi, fl->apsi, s->s0, s->sigma, AAh, AAl, K2, Kdot, uh, ul, c->dfa, c->dfa + N,
-                         fh, fl_, F.m, F.inv, c->partials, c->st);
+        gr::dfs_apsi(n, F.h2, fl->psi, fl->apsi, s->s0, s->sigma, AAh, AAl, K2, Kdot, uh, ul, c->dfa, c->dfa + N,
+                     fh, fl_, F.m, F.inv, sums_to(c, c->dscal, true), c->st);
     } else {
         // lap B^i = 2 d_j (alpha psi^-6 A^ij)  (Eqs. MDC-CF, MG-linear-2a)
         aij();
         if (c->w_fmt != 2) gr::dfs_weight(n, fl->psi, fl->apsi, wh, wl, c->st);
         c->w_fmt = 2;
-        g = gr::dfs_shift_rhs(n, 2.0 * (0.5 / c->h) * F.h2, A, wh, wl, eq - GR_BX, fld, uh, ul, fh, fl_,
-                              c->partials, c->st);
+        gr::dfs_shift_rhs(n, 2.0 * (0.5 / c->h) * F.h2, A, wh, wl, eq - GR_BX, fld, uh, ul, fh, fl_,
+                          sums_to(c, c->dscal, true), c->st);
     }
-    gr::finalize(c->partials, g, c->dscal, c->st);
     double a, q;
     gr_status st = read_scalars(c, &a, &q);
     if (st != GR_OK) return st;
@@ -753,53 +787,44 @@ void fmg32(gr_ctx *c, int kind32, int nu1, int nu2, float *uh, float *ul)
     }
 }
 
-gr_status norm64(gr_ctx *c, int kind, double rho, double ref, double *eps_nat, double *r)
+// The residual norms: queued here, read by read_norm.
+void norm64(gr_ctx *c, int kind, double rho, double *eps_nat)
 {
     Level &F = c->lev[c->nlev - 1];
-    const int64_t N = (int64_t)F.n * F.n * F.n;
-    int g = 0;
     timed(c, GR_PROF_NORM64, [&] {
-        g = gr::resid_norm<double>(kind, F.n, F.u, F.f, F.c0, F.c1, F.ih2, rho, c->partials, eps_nat, c->st);
+        gr::resid_norm<double>(kind, F.n, F.u, F.f, F.c0, F.c1, F.ih2, rho, sums_to(c, c->dscal, true), eps_nat, c->st);
     });
-    gr::finalize(c->partials, g, c->dscal, c->st);
-    double q;
-    gr_status st = read_scalars(c, &q, nullptr);
-    *r = std::sqrt(q / N) / ref;
-    return st;
 }
 
 // fine residual norm in double-float; with red != 0 also the first red
 // relaxation of the next correction cycle (into lev[fine].e)
-gr_status df_norm(gr_ctx *c, const EqInfo &in, double rho, bool red, double *r, const double *fshift = nullptr)
+void df_norm(gr_ctx *c, const EqInfo &in, double rho, bool red, const double *fshift = nullptr)
 {
     Level &F = c->lev[c->nlev - 1];
     const int64_t N = (int64_t)F.n * F.n * F.n;
-    int g = 0;
     timed(c, GR_PROF_MIXED_RESID, [&] {
-        g = gr::df_resid(in.kind, F.n, c->dfu, c->dfu + N, c->dff, c->dff + N, c->dfa, c->dfa + N, c->dfb,
-                         c->dfb + N, F.h2, rho, in.ref, F.r, F.m, F.inv, F.inv, red ? F.e : nullptr, c->partials,
-                         c->st, next_dir(c), fshift);
+        gr::df_resid(in.kind, F.n, c->dfu, c->dfu + N, c->dff, c->dff + N, c->dfa, c->dfa + N, c->dfb, c->dfb + N, F.h2,
+                     rho, in.ref, F.r, F.m, F.inv, F.inv, red ? F.e : nullptr, sums_to(c, c->dscal, true), c->st,
+                     next_dir(c), fshift);
     });
-    gr::finalize(c->partials, g, c->dscal, c->st);
-    double q;
-    gr_status st = read_scalars(c, &q, nullptr);
-    *r = std::sqrt(q / N);
-    return st;
 }
 
-gr_status mixed_norm(gr_ctx *c, const EqInfo &in, double rho, double *r)
+void mixed_norm(gr_ctx *c, const EqInfo &in, double rho)
 {
     Level &F = c->lev[c->nlev - 1];
-    const int64_t N = (int64_t)F.n * F.n * F.n;
-    int g = 0;
     timed(c, GR_PROF_MIXED_RESID, [&] {
-        g = gr::mixed_resid(in.kind, F.n, F.u, F.f, F.c0, F.c1, F.ih2, F.h2, rho, F.r, F.m, F.inv, c->partials,
-                            c->st);
+        gr::mixed_resid(in.kind, F.n, F.u, F.f, F.c0, F.c1, F.ih2, F.h2, rho, F.r, F.m, F.inv,
+                        sums_to(c, c->dscal, true), c->st);
     });
-    gr::finalize(c->partials, g, c->dscal, c->st);
-    double q;
-    gr_status st = read_scalars(c, &q, nullptr);
-    *r = std::sqrt(q / N) / in.ref;
+}
+
+// the relative residual of the last queued norm (back = 1: of the one before
+// it); ref = 1 for the double-float norm, which is relative already
+gr_status read_norm(gr_ctx *c, double ref, double *r, int back = 0)
+{
+    double q = NAN;
+    gr_status st = read_scalars(c, &q, nullptr, back);
+    *r = std::sqrt(q / ((double)c->n * c->n * c->n)) / ref;
     return st;
 }
 
@@ -1003,7 +1028,7 @@ gr_status patch_setup_eq(gr_ctx *c, int eq, const gr_opts *o, const EqInfo &in, 
     }
     double smean = 0.0;
     if (eq <= GR_VZ) {  // the base mean of s_i (the homogeneous background)
-        dsum(c, N0, s->s[eq]);
+        dsum(c, N0, s->s[eq], true);
         double a, q2;
         gr_status st = read_scalars(c, &a, &q2);
         if (st != GR_OK) return st;
@@ -1016,12 +1041,11 @@ gr_status patch_setup_eq(gr_ctx *c, int eq, const gr_opts *o, const EqInfo &in, 
         gr::PSetFld G;
         for (int q = 0; q < GR_NEQ; q++) G.g[q] = L.G[q];
         if (eq == GR_PSI) gr::patch_aij(L.n, 1.0 / L.h, G, L.A6, c->st);  // V and U are final from here on
-        const int g = gr::patch_setup(eq, L.n, 1.0 / L.h, S, G, L.A6, smean, K2, Kdot, L.f, L.c0, L.c1, c->partials,
-                                      c->st);
+        gr::Sums ref = sums_to(c, c->pdev + 16 + 2 * p);
+        ref.mapped = c->phost_dev + 16 + 2 * p;
+        gr::patch_setup(eq, L.n, 1.0 / L.h, S, G, L.A6, smean, K2, Kdot, L.f, L.c0, L.c1, ref, c->st);
         if (c->pdf) gr::patch_coef_df(in.kind, patch_view(c, p, in, rho), c->st);
-        gr::finalize(c->partials, g, c->pdev + 16 + 2 * p, c->st);
     }
-    gr::scalars_out(c->pdev + 16, c->phost_dev + 16, 2 * np, c->st);
     if (cudaStreamSynchronize(c->st) != cudaSuccess) return cuda_check("patch set-up");
     for (int p = 0; p < np; p++) {
         PatchLevel &L = c->pl[p];
@@ -1039,8 +1063,7 @@ gr_status patch_setup_eq(gr_ctx *c, int eq, const gr_opts *o, const EqInfo &in, 
     cudaMemsetAsync(c->pdev, 0, sizeof(double), c->st);  // lambda = 0
     if (in.poisson) {
         const gr::PBase B = base_view(c, fmt, rho);
-        const int g = gr::patch_sum_f_base(fmt, B, c->pl[0].o, c->pl[0].nc, c->partials, c->st);
-        gr::finalize(c->partials, g, c->pdev + 1, c->st);  // the original right-hand side over the covered cells
+        gr::patch_sum_f_base(fmt, B, c->pl[0].o, c->pl[0].nc, sums_to(c, c->pdev + 1), c->st);  // the original right-hand side over the covered cells
     }
     return cuda_check("patch set-up");
 }
@@ -1061,16 +1084,16 @@ void patch_down(gr_ctx *c, const EqInfo &in, int fmt, int nu, double rho)
             gr::patch_gs(in.kind, V, c->pdf, 0, c->st);
             gr::patch_gs(in.kind, V, c->pdf, 1, c->st);
         }
-        int g = gr::patch_resid(in.kind, V, c->pdf, L.eps, c->partials, c->st);
-        gr::finalize(c->partials, g, c->pdev + 32 + 2 * p, c->st);
+        gr::Sums norm = sums_to(c, c->pdev + 32 + 2 * p);  // for patch_norms: also to the host
+        norm.mapped = c->phost_dev + 32 + 2 * p;
+        gr::patch_resid(in.kind, V, c->pdf, L.eps, norm, c->st);
         gr::patch_restrict(V, c->pdf, L.eps, L.Ru, L.Re, c->st);
         if (p == 0) {
             const gr::PBase B = base_view(c, fmt, rho);
             gr::patch_inject_u_base(fmt, B, L.o, L.nc, L.Ru, c->st);
             gr::patch_gather_base(fmt, B, L.o, L.w, L.old, c->st);
-            g = gr::patch_inject_f_base(fmt, in.kind, B, L.o, L.nc, L.Re,
-                                        (fmt == gr::PB_DF && in.poisson) ? c->pdev : nullptr, c->partials, c->st);
-            gr::finalize(c->partials, g, c->pdev + 3, c->st);
+            gr::patch_inject_f_base(fmt, in.kind, B, L.o, L.nc, L.Re,
+                                    (fmt == gr::PB_DF && in.poisson) ? c->pdev : nullptr, sums_to(c, c->pdev + 3), c->st);
             gr::patch_reflux(fmt, B, gr::PPatch{}, V, c->pdf, L.o, c->h, L.flux, c->st);
             if (in.poisson) {
                 gr::patch_lambda(c->pdev + 1, L.flux, 6 * L.nc * L.nc, (double)N0, (double)L.nc * L.nc * L.nc,
@@ -1086,7 +1109,6 @@ void patch_down(gr_ctx *c, const EqInfo &in, int fmt, int nu, double rho)
             gr::patch_reflux(-1, gr::PBase{}, par, V, c->pdf, L.o, Q.h, L.flux, c->st);
         }
     }
-    gr::scalars_out(c->pdev + 32, c->phost_dev + 32, 2 * np, c->st);
 }
 
 // patches coarse to fine: the parent's correction P(u_new - u_old), fresh ghosts, nu sweeps
@@ -1158,13 +1180,15 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
             // the pair array (2N floats) fits the FP64 scratch level array
             cudaMemcpyAsync(F.ur, c->dfu, N * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
             cudaMemsetAsync(c->dfu, 0, N * sizeof(double), c->st);
-            st = df_norm(c, in, rho, false, &r_plain);
+            df_norm(c, in, rho, false);
+            st = read_norm(c, 1.0, &r_plain);
             if (st != GR_OK) return st;
             cudaMemcpyAsync(c->dfu, F.ur, N * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
         } else {
             cudaMemcpyAsync(F.ur, F.u, N * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
             cudaMemsetAsync(F.u, 0, N * sizeof(double), c->st);
-            st = norm64(c, in.kind, rho, in.ref, nullptr, &r_plain);
+            norm64(c, in.kind, rho, nullptr);
+            st = read_norm(c, in.ref, &r_plain);
             if (st != GR_OK) return st;
             cudaMemcpyAsync(F.u, F.ur, N * sizeof(double), cudaMemcpyDeviceToDevice, c->st);
         }
@@ -1185,11 +1209,14 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
     }
     double rlev[GR_MAX_PATCHES + 1] = {};
     // the base residual and, with patches, the largest of all levels' (rlev: each level's)
+    auto queue_norm = [&] {
+        if (dfm) df_norm(c, in, rho, red, (patches && in.poisson) ? c->pdev : nullptr);
+        else if (mixed) mixed_norm(c, in, rho);
+        else norm64(c, in.kind, rho, nullptr);
+    };
     auto fine_norm = [&](double *r) {
-        gr_status q;
-        if (dfm) q = df_norm(c, in, rho, red, r, (patches && in.poisson) ? c->pdev : nullptr);
-        else if (mixed) q = mixed_norm(c, in, rho, r);
-        else q = norm64(c, in.kind, rho, in.ref, nullptr, r);
+        queue_norm();
+        gr_status q = read_norm(c, dfm ? 1.0 : in.ref, r);
         rlev[0] = *r;
         if (q == GR_OK && patches) {
             patch_norms(c, rlev + 1);
@@ -1218,6 +1245,14 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
     if (res0) *res0 = r;
     int cyc = 0;
     if (!std::isfinite(r)) st = fail(GR_ERR_NONFINITE, "equation %d: initial residual is not finite", eq);
+    // While the residual is more than 1e4 above the tolerance the cycle after the
+    // next is certain to run (a V-cycle gains a factor of ten): it is queued
+    // without waiting for the next one's norm, which is read while it runs.
+    const bool ahead = !patches && !check && !c->prof_on;
+    bool unread = false;  // a norm is queued whose value r does not hold yet
+    auto finite = [&] {
+        if (st == GR_OK && !std::isfinite(r)) st = fail(GR_ERR_NONFINITE, "equation %d: residual not finite", eq);
+    };
     while (st == GR_OK && r > tol && cyc < max_cycles) {
         if (mixed) {
             if (in.kind == KPSI) restrict_coefs32(c);
@@ -1245,14 +1280,25 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
             });
             if (cells) *cells += patch_cells(c, o->nu1 + o->nu2);
         }
-        st = fine_norm(&r);
         cyc++;
         if (cells) *cells += per_cycle;
+        if (ahead) {
+            queue_norm();
+            if (unread) {
+                st = read_norm(c, dfm ? 1.0 : in.ref, &r, 1);
+                finite();
+            }
+            unread = st == GR_OK && r > 1e4 * tol && cyc < max_cycles;
+            if (!unread && st == GR_OK) st = read_norm(c, dfm ? 1.0 : in.ref, &r);
+            finite();
+            continue;
+        }
+        st = fine_norm(&r);
         if (st == GR_OK && check && cyc == 1 && !*rejected && !(r <= r_plain)) {
             use_plain_guess();
             st = fine_norm(&r);
         }
-        if (st == GR_OK && !std::isfinite(r)) st = fail(GR_ERR_NONFINITE, "equation %d: residual not finite", eq);
+        finite();
     }
     if (cycles) *cycles = cyc;
     if (res) *res = r;
@@ -1260,8 +1306,7 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
     // (the FP64 norm kernels leave the sum of u in dscal[1])
     if (dfm) {
         if (in.poisson) {
-            const int g = gr::dfs_pair_sum(N, c->dfu, c->dfu + N, c->partials, c->st);
-            gr::finalize(c->partials, g, c->dscal, c->st);
+            gr::dfs_pair_sum(N, c->dfu, c->dfu + N, sums_to(c, c->dscal), c->st);
         }
         gr::dfs_store(F.n, c->dfu, c->dfu + N, in.poisson ? c->dscal : nullptr, in.dev, field_ptr(fl, eq), c->st);
     } else {
@@ -1484,11 +1529,14 @@ gr_status gr_create(int n, double L, void *stream, gr_ctx **out)
     if (st == GR_OK) st = dalloc(c, &c->tmp, N);
     if (st == GR_OK) st = dalloc(c, &c->partials, 2 * kMaxRedBlocks);
     if (st == GR_OK) st = dalloc(c, &c->dscal, 16);
+    if (st == GR_OK) st = dalloc(c, &c->ticket, 1);
+    if (st == GR_OK) cudaMemsetAsync(c->ticket, 0, sizeof(unsigned), c->st);
     if (st == GR_OK && (cudaHostAlloc((void **)&c->hscal, 16 * sizeof(double), cudaHostAllocMapped) != cudaSuccess ||
                         cudaHostGetDevicePointer((void **)&c->hscal_dev, c->hscal, 0) != cudaSuccess)) {
         cudaGetLastError();
         st = fail(GR_ERR_NOMEM, "cudaHostAlloc (mapped scalars)");
     }
+    if (st == GR_OK) c->hscal[2] = c->hscal[6] = 0.0;
     if (st == GR_OK && (cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess)) {
         cudaGetLastError();
         st = fail(GR_ERR_CUDA, "cudaEventCreate");
@@ -1625,6 +1673,7 @@ gr_status gr_vcycle(gr_ctx *c, gr_eq eq, const gr_sources *s, gr_fields *fl, con
     base_only.npatch = 0;
     st = solve_eq(c, eq, s, fl, &base_only, rho, S_hat, -1.0, 1, nullptr, nullptr, &r, nullptr);
     if (res_after) *res_after = r;
+    if (cudaStreamSynchronize(c->st) != cudaSuccess && st == GR_OK) st = cuda_check("gr_vcycle");
     return st;
 }
 
@@ -1645,8 +1694,10 @@ gr_status gr_residual(gr_ctx *c, gr_eq eq, const gr_sources *s, const gr_fields 
     st = setup_eq(c, eq, s, fl, rho, S_hat, &in);
     if (st != GR_OK) return st;
     double r;
-    st = norm64(c, in.kind, rho, in.ref, res_field, &r);
+    norm64(c, in.kind, rho, res_field);
+    st = read_norm(c, in.ref, &r);
     if (rel_norm) *rel_norm = r;
+    if (cudaStreamSynchronize(c->st) != cudaSuccess && st == GR_OK) st = cuda_check("gr_residual");
     return st;
 }
 

@@ -135,7 +135,66 @@ constexpr int kBlock = 256;
 constexpr int kMaxRedBlocks = 152 * 16;  // blocks of the norm/mean reductions (16 per SM)
 constexpr int kCoarsestSweeps = 32;  // red-black sweeps on the 2^3 level
 
+// Where a kernel that reduces leaves its two sums: per-block partials, whose
+// sum (in a fixed order) the last block to finish writes to out[0], out[1]
+// and, if given, to mapped[0], mapped[1] (device alias of pinned host memory),
+// then seq to *flag (likewise).  A launch of its own for that sum cost 2.3 us
+// behind every residual, and another 2 us for the store to the host.  ticket:
+// a counter that is zero between launches; launches that share it must be
+// ordered.  partials == nullptr: no sums are wanted.
+struct Sums {
+    double *partials = nullptr, *out = nullptr;
+    unsigned *ticket = nullptr;
+    double *mapped = nullptr, *flag = nullptr;
+    double seq = 0.0;
+};
+
 #ifdef __CUDACC__
+// the end of a reducing kernel, by every thread of the block, after thread 0
+// wrote the block's partials
+__device__ __forceinline__ void last_block_sum(const Sums &S)
+{
+    __shared__ bool last;
+    __shared__ double la[kBlock / 32], lb[kBlock / 32];
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(S.ticket, gridDim.x - 1) == gridDim.x - 1;  // wraps to zero
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double a = 0.0, b = 0.0;
+    for (unsigned q = threadIdx.x; q < gridDim.x; q += kBlock) {
+        const double2 p = __ldcg(reinterpret_cast<const double2 *>(S.partials) + q);
+        a += p.x;
+        b += p.y;
+    }
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+    }
+    if (l == 0) la[w] = a, lb[w] = b;
+    __syncthreads();
+    if (w != 0) return;
+    a = l < kBlock / 32 ? la[l] : 0.0;
+    b = l < kBlock / 32 ? lb[l] : 0.0;
+    for (int o = kBlock / 64; o > 0; o >>= 1) {
+        a += __shfl_down_sync(0xffffffffu, a, o);
+        b += __shfl_down_sync(0xffffffffu, b, o);
+    }
+    if (l == 0) {
+        S.out[0] = a;
+        S.out[1] = b;
+        if (S.mapped) {
+            S.mapped[0] = a;
+            S.mapped[1] = b;
+            __threadfence_system();
+            if (S.flag) *(volatile double *)S.flag = S.seq;
+        }
+    }
+}
+
 // Block sums of a and b (blockDim.x == kBlock) into out[2 blockIdx.x + 0/1],
 // in a fixed order.
 __device__ __forceinline__ void block_sum2(double a, double b, double *out)
@@ -162,12 +221,20 @@ __device__ __forceinline__ void block_sum2(double a, double b, double *out)
     }
 }
 
+// Sums of a and b over the grid
+__device__ __forceinline__ void block_sum2(double a, double b, const Sums &S)
+{
+    block_sum2(a, b, S.partials);
+    last_block_sum(S);
+}
+
 // The same for FP32 inputs: warp sums in FP32 (for norms, where the rounding
 // of partial sums is harmless), the per-warp totals in FP64.  GB300's FP64
 // pipe is narrow enough that a full FP64 warp reduction per thread costs a
 // noticeable share of a memory-sized kernel.
-__device__ __forceinline__ void block_sum2f(float a, float b, double *out)
+__device__ __forceinline__ void block_sum2f(float a, float b, const Sums &S)
 {
+    double *const out = S.partials;
     __shared__ double sa[kBlock / 32], sb[kBlock / 32];
     for (int o = 16; o > 0; o >>= 1) {
         a += __shfl_down_sync(0xffffffffu, a, o);
@@ -188,6 +255,7 @@ __device__ __forceinline__ void block_sum2f(float a, float b, double *out)
         out[2 * blockIdx.x] = ta;
         out[2 * blockIdx.x + 1] = tb;
     }
+    last_block_sum(S);
 }
 #endif
 
@@ -248,18 +316,11 @@ void restrict_coef(int kind, int nf, const T *c0f, const T *c1f, T *c0c, T *c1c,
 template <typename T>
 void helm_invdiag(int n, const T *c0, T *c1, double h2, cudaStream_t st);
 
-// Block partial sums of eps^2 and of u over a level (split layout);
+// Sums of eps^2 and of u over a level (split layout);
 // eps_nat (may be null) receives eps in natural layout (double).
-// Partials: 2 doubles per block; returns the number of blocks.
 template <typename T>
-int resid_norm(int kind, int n, const T *u, const T *f, const T *c0, const T *c1, double ih2, double rho,
-               double *partials, double *eps_nat, cudaStream_t st);
-// out[0] = sum of partials[2b], out[1] = sum of partials[2b + 1].
-void finalize(const double *partials, int nblk, double *out, cudaStream_t st);
-// dst_mapped[0 .. cnt) = src[0 .. cnt) (cnt <= 32): dst_mapped is the device
-// alias of pinned host memory allocated with cudaHostAllocMapped.
-void scalars_out(const double *src, double *dst_mapped, int cnt, cudaStream_t st);
-
+void resid_norm(int kind, int n, const T *u, const T *f, const T *c0, const T *c1, double ih2, double rho,
+                const Sums &sums, double *eps_nat, cudaStream_t st);
 // The FP32 correction cycle's levels coarse_tail_n()^3 .. 2^3 in one thread
 // block (shared memory): e/r/m/inv of levels 2^3, 4^3, 8^3, 16^3 (index 0 =
 // 2^3); e and r of the top tail level in and e out; h2 per level.
@@ -301,8 +362,8 @@ void tail64(int kind, int top, double *u, const double *f, const double *const *
 // ---- mixed precision -------------------------------------------------------
 // FP64 residual on the fine level; writes r32 = -eps (split), and for KPSI
 // the Jacobian coefficient m32 = -dN/du > 0 and its inverse diagonal inv32.
-int mixed_resid(int kind, int n, const double *u, const double *f, const double *c0, const double *c1, double ih2,
-                double h2, double rho, float *r32, float *m32, float *inv32, double *partials, cudaStream_t st);
+void mixed_resid(int kind, int n, const double *u, const double *f, const double *c0, const double *c1, double ih2,
+                double h2, double rho, float *r32, float *m32, float *inv32, const Sums &sums, cudaStream_t st);
 // u64 += e32 (split layout).
 void mixed_update(int n, double *u, const float *e, cudaStream_t st);
 // c32 = (float) c64.
@@ -315,11 +376,10 @@ void to_float(int64_t cnt, const double *a, float *b, cudaStream_t st);
 // premultiplied by h^2 (KPOISSON, KHELM: h^2 f, h^2 m; KPSI: f' = h^2 f,
 // a' = 2 pi h^2 s0, b' = h^2 AA / 8).  When e32 is not null it also writes the
 // first red relaxation of the correction cycle from e = 0 (inv_in: the KHELM
-// inverse diagonal).  Partials: block sums of (eps/ref)^2.  Returns the block
-// count.
-int df_resid(int kind, int n, const float *uh, const float *ul, const float *fh, const float *fl, const float *ah,
+// inverse diagonal).  Sums: of (eps/ref)^2.
+void df_resid(int kind, int n, const float *uh, const float *ul, const float *fh, const float *fl, const float *ah,
              const float *al, const float *bh, const float *bl, double h2, double rho, double ref, float *r32,
-             float *m32, float *inv32, const float *inv_in, float *e32, double *partials, cudaStream_t st, int rev = 0,
+             float *m32, float *inv32, const float *inv_in, float *e32, const Sums &sums, cudaStream_t st, int rev = 0,
              const double *fshift = nullptr);
 void df_update(int n, float *uh, float *ul, const float *e, cudaStream_t st);
 // last black pass of the FP32 correction cycle (KPOISSON or KHELM, n >= 8)
@@ -330,32 +390,31 @@ void df_black_update(int kind, int n, const float *e, const float *r, const floa
 // ---- double-float set-up and write-back (df_setup.cu) -----------------------
 // Natural FP64 inputs -> split-layout hi/lo pairs, right-hand sides and
 // coefficients premultiplied by h^2 as df_resid takes them (the callers pass
-// the scales with h^2 folded in).  The int-returning ones
-// leave block partials (sum, sum of squares of the high parts) of the
-// quantity named and return the block count for finalize().
-int dfs_sum(int64_t cnt, const double *a, double *partials, cudaStream_t st);                      // a
-int dfs_pair_sum(int64_t cnt, const float *h, const float *l, double *partials, cudaStream_t st);  // h + l
-// f = scale (s - sum[0]/n^3), u = fld; partials of f
-int dfs_mean_rhs(int n, const double *s, const double *sum, double scale, const double *fld, float *uh, float *ul,
-                 float *fh, float *fl, double *partials, cudaStream_t st);
-// f = scale sum_l (F_l(+l) - F_l(-l)), u = fld; partials of f
-int dfs_div_rhs(int n, double scale, const double *Fx, const double *Fy, const double *Fz, const double *fld,
-                float *uh, float *ul, float *fh, float *fl, double *partials, cudaStream_t st);
-// f = scale sum_l ((A^{comp l} w)(+l) - (A^{comp l} w)(-l)), u = fld; partials of f
-int dfs_shift_rhs(int n, double scale, const float *A, const float *wh, const float *wl, int comp, const double *fld,
-                  float *uh, float *ul, float *fh, float *fl, double *partials, cudaStream_t st);
+// the scales with h^2 folded in).  sums: sum and sum of squares of the high
+// parts of the quantity named.
+void dfs_sum(int64_t cnt, const double *a, const Sums &sums, cudaStream_t st);                      // a
+void dfs_pair_sum(int64_t cnt, const float *h, const float *l, const Sums &sums, cudaStream_t st);  // h + l
+// f = scale (s - sum[0]/n^3), u = fld; sums of f
+void dfs_mean_rhs(int n, const double *s, const double *sum, double scale, const double *fld, float *uh, float *ul,
+                 float *fh, float *fl, const Sums &sums, cudaStream_t st);
+// f = scale sum_l (F_l(+l) - F_l(-l)), u = fld; sums of f
+void dfs_div_rhs(int n, double scale, const double *Fx, const double *Fy, const double *Fz, const double *fld,
+                float *uh, float *ul, float *fh, float *fl, const Sums &sums, cudaStream_t st);
+// f = scale sum_l ((A^{comp l} w)(+l) - (A^{comp l} w)(-l)), u = fld; sums of f
+void dfs_shift_rhs(int n, double scale, const float *A, const float *wh, const float *wl, int comp, const double *fld,
+                  float *uh, float *ul, float *fh, float *fl, const Sums &sums, cudaStream_t st);
 // A_ij (12 n^3 floats: component c hi at A + 2c n^3, lo at A + (2c+1) n^3) and AA pairs, natural layout;
 // scratch: four arrays of 2 n^3 floats for the pairs of V_x, V_y, V_z, U
 void dfs_aij(int n, double inv2h, double ih2, const double *Vx, const double *Vy, const double *Vz, const double *U,
              float *const scratch[4], float *A, float *AAh, float *AAl, cudaStream_t st);
-// psi: u = psi - 1, a = 2 pi h^2 s0, b = h^2 AA / 8, f = 0; partials of s0
-int dfs_psi(int n, double h2, const double *psi, const double *s0, const float *AAh, const float *AAl, float *uh,
-            float *ul, float *ah, float *al, float *bh, float *bl, float *fh, float *fl, double *partials,
+// psi: u = psi - 1, a = 2 pi h^2 s0, b = h^2 AA / 8, f = 0; sums of s0
+void dfs_psi(int n, double h2, const double *psi, const double *s0, const float *AAh, const float *AAl, float *uh,
+            float *ul, float *ah, float *al, float *bh, float *bl, float *fh, float *fl, const Sums &sums,
             cudaStream_t st);
-// alpha psi: u = alpha psi - 1, a = h^2 m, f = h^2 (m - psi^5 Kdot), m32, inv32; partials of psi^5 Kdot
-int dfs_apsi(int n, double h2, const double *psi, const double *apsi, const double *s0, const double *sig,
+// alpha psi: u = alpha psi - 1, a = h^2 m, f = h^2 (m - psi^5 Kdot), m32, inv32; sums of psi^5 Kdot
+void dfs_apsi(int n, double h2, const double *psi, const double *apsi, const double *s0, const double *sig,
              const float *AAh, const float *AAl, double K2, double Kdot, float *uh, float *ul, float *ah, float *al,
-             float *fh, float *fl, float *m32, float *inv32, double *partials, cudaStream_t st);
+             float *fh, float *fl, float *m32, float *inv32, const Sums &sums, cudaStream_t st);
 // w = alpha psi psi^-7 pairs, natural layout
 void dfs_weight(int n, const double *psi, const double *apsi, float *wh, float *wl, cudaStream_t st);
 // out (natural) = hi + lo - sum[0]/n^3 (sum may be null) + (dev ? 1 : 0)
@@ -368,8 +427,8 @@ void deposit(int n, double L, int64_t np, const double *x, const double *u, doub
 // particles arriving in chunks
 void deposit_add(int n, double L, int64_t np, const double *x, const double *u, double mass, double *s0, double *sx,
                  double *sy, double *sz, double *sig, cudaStream_t st);
-// Partial sums of a and a^2 over cnt doubles; returns the block count.
-int sum_sq(int64_t cnt, const double *a, double *partials, cudaStream_t st);
+// Sums of a and a^2 over cnt doubles.
+void sum_sq(int64_t cnt, const double *a, const Sums &sums, cudaStream_t st);
 // a[i] = scale * (a[i] - s[0] / cnt_total), s a device scalar (a sum).
 void scale_sub_mean(int64_t cnt, double *a, const double *sum, double inv_cnt, double scale, cudaStream_t st);
 // natural -> split with a shift: split = nat + shift; split -> natural:
@@ -480,12 +539,12 @@ void patch_gather_patch(const PPatch &par, bool pdf, const int o[3], int w, doub
 // ghosts of the unknown = P(win); with d (or its FP32 copy d32 for pdf), the interior += P(d)
 void patch_interp(const PPatch &P, bool pdf, const double *win, const double *d, const float *d32, cudaStream_t st);
 void patch_gs(int kind, const PPatch &P, bool pdf, int color, cudaStream_t st);
-int patch_resid(int kind, const PPatch &P, bool pdf, double *eps, double *partials, cudaStream_t st);
+void patch_resid(int kind, const PPatch &P, bool pdf, double *eps, const Sums &sums, cudaStream_t st);
 void patch_restrict(const PPatch &P, bool pdf, const double *eps, double *Ru, double *Re, cudaStream_t st);
 void patch_inject_u_base(int fmt, const PBase &B, const int o[3], int nc, const double *Ru, cudaStream_t st);
-int patch_inject_f_base(int fmt, int kind, const PBase &B, const int o[3], int nc, const double *Re, const double *lam,
-                        double *partials, cudaStream_t st);
-int patch_sum_f_base(int fmt, const PBase &B, const int o[3], int nc, double *partials, cudaStream_t st);
+void patch_inject_f_base(int fmt, int kind, const PBase &B, const int o[3], int nc, const double *Re, const double *lam,
+                        const Sums &sums, cudaStream_t st);
+void patch_sum_f_base(int fmt, const PBase &B, const int o[3], int nc, const Sums &sums, cudaStream_t st);
 void patch_inject_u_patch(const PPatch &par, bool pdf, const int o[3], int nc, const double *Ru, cudaStream_t st);
 void patch_inject_f_patch(int kind, const PPatch &par, bool pdf, const int o[3], int nc, const double *Re,
                           cudaStream_t st);
@@ -500,8 +559,8 @@ void patch_u_store(const PPatch &P, bool pdf, double *out, double *keep, double 
 void patch_coef_df(int kind, const PPatch &P, cudaStream_t st);
 // A_ij of the ghosted V, U on the interior and first ghost layer (six ghosted arrays)
 void patch_aij(int n, double nh, const PSetFld &G, double *A6, cudaStream_t st);
-int patch_setup(int eq, int n, double nh, const PSetSrc &S, const PSetFld &G, const double *A6, double smean,
-                double K2, double Kdot, double *f, double *c0, double *c1, double *partials, cudaStream_t st);
+void patch_setup(int eq, int n, double nh, const PSetSrc &S, const PSetFld &G, const double *A6, double smean,
+                double K2, double Kdot, double *f, double *c0, double *c1, const Sums &sums, cudaStream_t st);
 
 // Three FP32 colour passes of the correction equation (KPOISSON, KHELM) in
 // one pass over memory: colour c1 from the other colour of ein, then the other

@@ -747,7 +747,7 @@ __global__ void k_helm_invdiag(int64_t cnt, const T *__restrict__ c0, T *__restr
 template <typename T, int KIND>
 __global__ void __launch_bounds__(kBlock)
     k_resid_norm(int lgn, const T *__restrict__ u, const T *__restrict__ f, const T *__restrict__ c0,
-                 const T *__restrict__ c1, T ih2, T rho, double *__restrict__ partials, double *__restrict__ eps_nat)
+                 const T *__restrict__ c1, T ih2, T rho, const Sums sums, double *__restrict__ eps_nat)
 {
     pdl_begin();
     const int64_t ncells = (int64_t)1 << (3 * lgn);
@@ -761,30 +761,7 @@ __global__ void __launch_bounds__(kBlock)
         su += (double)u[t];
         if (eps_nat) eps_nat[((((int64_t)i << lgn) + j) << lgn) + k] = e;
     }
-    block_sum2(s2, su, partials);
-}
-
-__global__ void __launch_bounds__(kBlock) k_finalize(const double *__restrict__ partials, int nblk,
-                                                     double *__restrict__ out)
-{
-    pdl_begin();
-    // one block, fixed summation order: out[0], out[1] = block_sum2's slots of block 0
-    double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < nblk; q += kBlock) {
-        a += partials[2 * q];
-        b += partials[2 * q + 1];
-    }
-    block_sum2(a, b, out);
-}
-
-// cnt (<= 32) doubles from device memory to host-mapped pinned memory: the
-// host reads them after a stream synchronisation without a copy-engine
-// transfer, which would queue behind large copies in flight on other streams
-__global__ void k_scalars_out(const double *__restrict__ src, double *dst, int cnt)
-{
-    pdl_begin();
-    if ((int)threadIdx.x < cnt) dst[threadIdx.x] = src[threadIdx.x];
-    __threadfence_system();
+    block_sum2(s2, su, sums);
 }
 
 // ---------------------------------------------------------------- mixed precision
@@ -792,7 +769,7 @@ template <int KIND>
 __global__ void __launch_bounds__(kBlock)
     k_mixed_resid(int lgn, const double *__restrict__ u, const double *__restrict__ f, const double *__restrict__ c0,
                   const double *__restrict__ c1, double ih2, double h2, double rho, float *__restrict__ r32,
-                  float *__restrict__ m32, float *__restrict__ inv32, double *__restrict__ partials)
+                  float *__restrict__ m32, float *__restrict__ inv32, const Sums sums)
 {
     pdl_begin();
     const int64_t ncells = (int64_t)1 << (3 * lgn);
@@ -813,7 +790,7 @@ __global__ void __launch_bounds__(kBlock)
             inv32[t] = 1.0f / (6.0f + (float)h2 * mf);
         }
     }
-    block_sum2(s2, su, partials);
+    block_sum2(s2, su, sums);
 }
 
 __global__ void k_mixed_update(int64_t cnt, double *__restrict__ u, const float *__restrict__ e)
@@ -985,49 +962,35 @@ void helm_invdiag(int n, const T *c0, T *c1, double h2, cudaStream_t st)
     GR_LAUNCH((k_helm_invdiag<T>), grid_for(cnt), kBlock, st, cnt, c0, c1, (T)h2);
 }
 
-static int red_grid(int64_t cnt)
-{
-    int g = grid_for(cnt);
-    return g > kMaxRedBlocks ? kMaxRedBlocks : g;
-}
-
+// (reductions take one full wave: every block ends with an atomic on the shared
+// ticket, and 2432 of them in turn cost more than a second launch would)
 template <typename T>
-int resid_norm(int kind, int n, const T *u, const T *f, const T *c0, const T *c1, double ih2, double rho,
-               double *partials, double *eps_nat, cudaStream_t st)
+void resid_norm(int kind, int n, const T *u, const T *f, const T *c0, const T *c1, double ih2, double rho,
+                const Sums &sums, double *eps_nat, cudaStream_t st)
 {
     const int lgn = log2i(n);
-    const int g = red_grid((int64_t)n * n * n);
-    if (kind == KPOISSON)
-        GR_LAUNCH((k_resid_norm<T, KPOISSON>), g, kBlock, st, lgn, u, f, c0, c1, (T)ih2, (T)rho, partials, eps_nat);
-    else if (kind == KHELM)
-        GR_LAUNCH((k_resid_norm<T, KHELM>), g, kBlock, st, lgn, u, f, c0, c1, (T)ih2, (T)rho, partials, eps_nat);
-    else
-        GR_LAUNCH((k_resid_norm<T, KPSI>), g, kBlock, st, lgn, u, f, c0, c1, (T)ih2, (T)rho, partials, eps_nat);
-    return g;
+    const int64_t cnt = (int64_t)n * n * n;
+#define GR_RN(K)                                                                                                    \
+    GR_LAUNCH((k_resid_norm<T, K>), wave_grid(k_resid_norm<T, K>, cnt), kBlock, st, lgn, u, f, c0, c1, (T)ih2, (T)rho, \
+              sums, eps_nat)
+    if (kind == KPOISSON) GR_RN(KPOISSON);
+    else if (kind == KHELM) GR_RN(KHELM);
+    else GR_RN(KPSI);
+#undef GR_RN
 }
 
-void finalize(const double *partials, int nblk, double *out, cudaStream_t st)
-{
-    GR_LAUNCH(k_finalize, 1, kBlock, st, partials, nblk, out);
-}
-
-void scalars_out(const double *src, double *dst_mapped, int cnt, cudaStream_t st)
-{
-    GR_LAUNCH(k_scalars_out, 1, 32, st, src, dst_mapped, cnt);
-}
-
-int mixed_resid(int kind, int n, const double *u, const double *f, const double *c0, const double *c1, double ih2,
-                double h2, double rho, float *r32, float *m32, float *inv32, double *partials, cudaStream_t st)
+void mixed_resid(int kind, int n, const double *u, const double *f, const double *c0, const double *c1, double ih2,
+                 double h2, double rho, float *r32, float *m32, float *inv32, const Sums &sums, cudaStream_t st)
 {
     const int lgn = log2i(n);
-    const int g = red_grid((int64_t)n * n * n);
-    if (kind == KPOISSON)
-        GR_LAUNCH((k_mixed_resid<KPOISSON>), g, kBlock, st, lgn, u, f, c0, c1, ih2, h2, rho, r32, m32, inv32, partials);
-    else if (kind == KHELM)
-        GR_LAUNCH((k_mixed_resid<KHELM>), g, kBlock, st, lgn, u, f, c0, c1, ih2, h2, rho, r32, m32, inv32, partials);
-    else
-        GR_LAUNCH((k_mixed_resid<KPSI>), g, kBlock, st, lgn, u, f, c0, c1, ih2, h2, rho, r32, m32, inv32, partials);
-    return g;
+    const int64_t cnt = (int64_t)n * n * n;
+#define GR_MR(K)                                                                                                 \
+    GR_LAUNCH((k_mixed_resid<K>), wave_grid(k_mixed_resid<K>, cnt), kBlock, st, lgn, u, f, c0, c1, ih2, h2, rho, r32, \
+              m32, inv32, sums)
+    if (kind == KPOISSON) GR_MR(KPOISSON);
+    else if (kind == KHELM) GR_MR(KHELM);
+    else GR_MR(KPSI);
+#undef GR_MR
 }
 
 void mixed_update(int n, double *u, const float *e, cudaStream_t st)
@@ -1050,8 +1013,8 @@ void to_float(int64_t cnt, const double *a, float *b, cudaStream_t st)
     template void coarsest<T>(int, T *, T *, const T *, const T *, double, double, double, cudaStream_t);           \
     template void restrict_coef<T>(int, int, const T *, const T *, T *, T *, double, cudaStream_t);                \
     template void helm_invdiag<T>(int, const T *, T *, double, cudaStream_t);                                      \
-    template int resid_norm<T>(int, int, const T *, const T *, const T *, const T *, double, double, double *,     \
-                               double *, cudaStream_t);
+    template void resid_norm<T>(int, int, const T *, const T *, const T *, const T *, double, double,              \
+                                const Sums &, double *, cudaStream_t);
 GR_INST(double)
 GR_INST(float)
 
