@@ -307,18 +307,6 @@ void deposit_add(int n, double L, int64_t np, const double *x, const double *u, 
     GR_LAUNCH(k_deposit, g, kBlock, st, log2i(n), 1.0 / h, np, x, u, q, s0, sx, sy, sz, sig);
 }
 
-void deposit(int n, double L, int64_t np, const double *x, const double *u, double mass, double *s0, double *sx,
-             double *sy, double *sz, double *sig, cudaStream_t st)
-{
-    const size_t bytes = (size_t)n * n * n * sizeof(double);
-    cudaMemsetAsync(s0, 0, bytes, st);
-    cudaMemsetAsync(sx, 0, bytes, st);
-    cudaMemsetAsync(sy, 0, bytes, st);
-    cudaMemsetAsync(sz, 0, bytes, st);
-    cudaMemsetAsync(sig, 0, bytes, st);
-    deposit_add(n, L, np, x, u, mass, s0, sx, sy, sz, sig, st);
-}
-
 void sum_sq(int64_t cnt, const double *a, const Sums &sums, cudaStream_t st)
 {
     const int g = wave_grid(k_sum_sq, cnt);

@@ -1368,6 +1368,29 @@ gr_status ensure_copy_stream(gr_ctx *c)
     return GR_OK;
 }
 
+// The sources zeroed (first) and np particles added, over tiles where they
+// fill the grid (psi null: the plain deposit)
+void deposit_device(gr_ctx *c, int64_t np, const double *x, const double *u, double mass, const double *psi,
+                    const gr_sources *out, bool first)
+{
+    if (first) {
+        const size_t bytes = (size_t)c->n * c->n * c->n * sizeof(double);
+        double *f[5] = {out->s0, out->s[0], out->s[1], out->s[2], out->sigma};
+        for (int k = 0; k < 5; k++) cudaMemsetAsync(f[k], 0, bytes, c->st);
+    }
+    const size_t scratch = 6 * (size_t)c->n * c->n * c->n * sizeof(double);  // A_ij, which a solve makes anew
+    if (gr::deposit_tiles_fit(c->n, c->L, np, mass, psi != nullptr, scratch)) {
+        c->a_fmt = 0;
+        gr::deposit_tiles(c->n, c->L, np, np, x, u, mass, psi, out->s0, out->s[0], out->s[1], out->s[2], out->sigma,
+                          c->A6, scratch, !first, c->st);
+    } else if (psi) {
+        gr::deposit_metric_add(c->n, c->L, np, x, u, mass, psi, out->s0, out->s[0], out->s[1], out->s[2], out->sigma,
+                               c->st);
+    } else {
+        gr::deposit_add(c->n, c->L, np, x, u, mass, out->s0, out->s[0], out->s[1], out->s[2], out->sigma, c->st);
+    }
+}
+
 // Deposit from host arrays: chunks of particles go through two staging
 // buffers; chunk i's six copies (x and u, three components each) run on the
 // copy stream while chunk i-1 deposits on the context's stream.
@@ -1384,9 +1407,6 @@ gr_status deposit_from_host(gr_ctx *c, int64_t np, const double *x, const double
         }
         c->stage_cap = chunk;
     }
-    const size_t bytes = (size_t)c->n * c->n * c->n * sizeof(double);
-    double *f[5] = {out->s0, out->s[0], out->s[1], out->s[2], out->sigma};
-    for (int k = 0; k < 5; k++) cudaMemsetAsync(f[k], 0, bytes, c->st);
     // the staging buffers may still be read by the previous call's last chunks
     for (int b = 0; b < 2; b++) cudaEventRecord(c->used[b], c->st);
     int b = 0;
@@ -1400,7 +1420,7 @@ gr_status deposit_from_host(gr_ctx *c, int64_t np, const double *x, const double
         }
         cudaEventRecord(c->ready[b], c->cs);
         cudaStreamWaitEvent(c->st, c->ready[b], 0);
-        gr::deposit_add(c->n, c->L, m, xs, us, mass, out->s0, out->s[0], out->s[1], out->s[2], out->sigma, c->st);
+        deposit_device(c, m, xs, us, mass, nullptr, out, p0 == 0);
         cudaEventRecord(c->used[b], c->st);
     }
     return GR_OK;
@@ -1563,7 +1583,7 @@ gr_status gr_deposit(gr_ctx *c, int64_t np, const double *x, const double *u, do
         gr_status st = deposit_from_host(c, np, x, u, mass, out);
         if (st != GR_OK) return st;
     } else {
-        gr::deposit(c->n, c->L, np, x, u, mass, out->s0, out->s[0], out->s[1], out->s[2], out->sigma, c->st);
+        deposit_device(c, np, x, u, mass, nullptr, out, true);
     }
     c->rho_dep = mass * (double)np / (c->L * c->L * c->L);
     return cuda_check("gr_deposit");
@@ -1802,7 +1822,7 @@ gr_status gr_deposit_metric(gr_ctx *c, int64_t np, const double *x, const double
         return fail(GR_ERR_ARG, "gr_deposit_metric takes device particle arrays");
     if (!psi) return gr_deposit(c, np, x, u, mass, out);
     if (host_memory(psi)) return fail(GR_ERR_ARG, "psi must be device memory");
-    gr::deposit_metric(c->n, c->L, np, x, u, mass, psi, out->s0, out->s[0], out->s[1], out->s[2], out->sigma, c->st);
+    deposit_device(c, np, x, u, mass, psi, out, true);
     c->rho_dep = mass * (double)np / (c->L * c->L * c->L);
     return cuda_check("gr_deposit_metric");
 }

@@ -421,12 +421,19 @@ void dfs_weight(int n, const double *psi, const double *apsi, float *wh, float *
 void dfs_store(int n, const float *uh, const float *ul, const double *sum, int dev, double *out, cudaStream_t st);
 
 // ---- sources, coefficients, layouts (field_kernels.cu) ---------------------
-void deposit(int n, double L, int64_t np, const double *x, const double *u, double mass, double *s0, double *sx,
-             double *sy, double *sz, double *sig, cudaStream_t st);
-// the deposit kernel alone, adding to the five arrays (no zeroing): for
-// particles arriving in chunks
+// the deposit kernel, one thread per particle, adding to the five arrays (no zeroing)
 void deposit_add(int n, double L, int64_t np, const double *x, const double *u, double mass, double *s0, double *sx,
                  double *sy, double *sz, double *sig, cudaStream_t st);
+// The same over tiles of 8^3 cells (deposit_tiles.cu), psi null: the plain
+// deposit, else with the metric's Lorentz factor; x, u: [3][stride], np of them;
+// adds to the five arrays (add: other launches have added to them already;
+// otherwise they hold zeros).  scratch: device memory.  deposit_tiles_fit: the
+// particles fill the grid well enough for it, the charge mass / h^3 is in its
+// range and the scratch suffices.
+bool deposit_tiles_fit(int n, double L, int64_t np, double mass, bool metric, size_t scratch);
+void deposit_tiles(int n, double L, int64_t np, int64_t stride, const double *x, const double *u, double mass,
+                   const double *psi, double *s0, double *sx, double *sy, double *sz, double *sig, void *scratch,
+                   size_t bytes, bool add, cudaStream_t st);
 // Sums of a and a^2 over cnt doubles.
 void sum_sq(int64_t cnt, const double *a, const Sums &sums, cudaStream_t st);
 // a[i] = scale * (a[i] - s[0] / cnt_total), s a device scalar (a sum).
@@ -466,8 +473,9 @@ void particle_fields(int n, double L, const double *psi, const double *apsi, con
 void particle_update(int n, double L, int64_t np, double *x, double *u, const float *rec, double dt, int flags,
                      cudaStream_t st);
 // The deposit with W = sqrt(1 + psi^-4 |u|^2), psi interpolated at the particle.
-void deposit_metric(int n, double L, int64_t np, const double *x, const double *u, double mass, const double *psi,
-                    double *s0, double *sx, double *sy, double *sz, double *sig, cudaStream_t st);
+// One thread per particle, adding to the five arrays.
+void deposit_metric_add(int n, double L, int64_t np, const double *x, const double *u, double mass, const double *psi,
+                        double *s0, double *sx, double *sy, double *sz, double *sig, cudaStream_t st);
 
 // ---- code units (codeunits.cu) ----------------------------------------------
 struct CuPtrs {

@@ -311,15 +311,9 @@ void particle_update(int n, double L, int64_t np, double *x, double *u, const fl
               (float)(0.5 * dt), dt, flags);
 }
 
-void deposit_metric(int n, double L, int64_t np, const double *x, const double *u, double mass, const double *psi,
-                    double *s0, double *sx, double *sy, double *sz, double *sig, cudaStream_t st)
+void deposit_metric_add(int n, double L, int64_t np, const double *x, const double *u, double mass, const double *psi,
+                        double *s0, double *sx, double *sy, double *sz, double *sig, cudaStream_t st)
 {
-    const size_t bytes = (size_t)n * n * n * sizeof(double);
-    cudaMemsetAsync(s0, 0, bytes, st);
-    cudaMemsetAsync(sx, 0, bytes, st);
-    cudaMemsetAsync(sy, 0, bytes, st);
-    cudaMemsetAsync(sz, 0, bytes, st);
-    cudaMemsetAsync(sig, 0, bytes, st);
     if (np <= 0) return;
     const double h = L / n;
     const int64_t blocks = (np + kBlock - 1) / kBlock;
