@@ -170,66 +170,89 @@ __global__ void __launch_bounds__(kBlock)
     }
 }
 
-// A_ij of Eq. Aij-discrete-2 (xx yy zz xy xz yz, natural) and AA = A_ij A^ij
+// A_ij of Eq. Aij-discrete-2 (xx yy zz xy xz yz, natural) and AA = A_ij A^ij.
+// FP64 issue is the bound, so the sums are formed on unscaled differences, in
+// units of 1/2h (r = 2 (1/h^2) / (1/2h), the second derivatives' factor in
+// those units), and scaled once: 45 operations per cell for AA and 6 more for
+// the stored A_ij, where scaling every derivative took 65.  256^3: 1.97 -> 1.42
+// ms without the stores (45 operations at the measured FP64 rate: 1.43).
+template <bool STORE>
 __global__ void __launch_bounds__(kBlock)
-    k_aij_aa(int lgn, double inv2h, double ih2, const double *__restrict__ Vx, const double *__restrict__ Vy,
+    k_aij_aa(int lgn, double inv2h, double r, const double *__restrict__ Vx, const double *__restrict__ Vy,
              const double *__restrict__ Vz, const double *__restrict__ U, double *__restrict__ A,
              double *__restrict__ AA)
 {
     pdl_begin();
     const int64_t cnt = (int64_t)1 << (3 * lgn);
     const int m = (1 << lgn) - 1;
-    const double *V[3] = {Vx, Vy, Vz};
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
-        const int k = (int)(t & m), j = (int)((t >> lgn) & m), i = (int)(t >> (2 * lgn));
-        double D[3][3];
+    const double r4 = 0.25 * r, sc = inv2h * inv2h;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < (int)cnt; t += gridDim.x * blockDim.x) {
+        const int k = t & m, j = (t >> lgn) & m, i = t >> (2 * lgn);
+        const int kp = (k + 1) & m, km = (k - 1) & m;
+        // rows (i, j), (i +- 1, j), (i, j +- 1) and the four diagonal ones
+        const int jo = j << lgn, jp = ((j + 1) & m) << lgn, jm = ((j - 1) & m) << lgn;
+        const int io = i << (2 * lgn), ip = ((i + 1) & m) << (2 * lgn), im = ((i - 1) & m) << (2 * lgn);
+        const double *const V[3] = {Vx, Vy, Vz};
+        double D[3][3];  // D[a][l] = V_l(+a) - V_l(-a)
 #pragma unroll
-        for (int a = 0; a < 3; a++)
-#pragma unroll
-            for (int l = 0; l < 3; l++) D[a][l] = (at(V[l], lgn, i, j, k, a, 1) - at(V[l], lgn, i, j, k, a, -1)) * inv2h;
-        const double divV = D[0][0] + D[1][1] + D[2][2];
+        for (int l = 0; l < 3; l++) {
+            D[0][l] = V[l][ip + jo + k] - V[l][im + jo + k];
+            D[1][l] = V[l][io + jp + k] - V[l][io + jm + k];
+            D[2][l] = V[l][io + jo + kp] - V[l][io + jo + km];
+        }
         const double u0 = U[t];
+        const double S[3] = {U[ip + jo + k] + U[im + jo + k], U[io + jp + k] + U[io + jm + k],
+                             U[io + jo + kp] + U[io + jo + km]};
+        const double c = fma(-2.0 * r, u0, -0.5 * (D[0][0] + D[1][1] + D[2][2]));
         double Ad[3], Ao[3];
 #pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const double Uaa = (at(U, lgn, i, j, k, a, 1) - 2.0 * u0 + at(U, lgn, i, j, k, a, -1)) * ih2;
-            Ad[a] = 2.0 * D[a][a] - 0.5 * divV + 2.0 * Uaa;
-        }
-        const int ip = (i + 1) & m, im = (i - 1) & m, jp = (j + 1) & m, jm = (j - 1) & m, kp = (k + 1) & m,
-                  km = (k - 1) & m;
-        const double Uxy = (U[nidx(lgn, ip, jp, k)] + U[nidx(lgn, im, jm, k)] - U[nidx(lgn, im, jp, k)] -
-                            U[nidx(lgn, ip, jm, k)]) * (0.25 * ih2);
-        const double Uxz = (U[nidx(lgn, ip, j, kp)] + U[nidx(lgn, im, j, km)] - U[nidx(lgn, im, j, kp)] -
-                            U[nidx(lgn, ip, j, km)]) * (0.25 * ih2);
-        const double Uyz = (U[nidx(lgn, i, jp, kp)] + U[nidx(lgn, i, jm, km)] - U[nidx(lgn, i, jm, kp)] -
-                            U[nidx(lgn, i, jp, km)]) * (0.25 * ih2);
-        Ao[0] = D[0][1] + D[1][0] + 2.0 * Uxy;
-        Ao[1] = D[0][2] + D[2][0] + 2.0 * Uxz;
-        Ao[2] = D[1][2] + D[2][1] + 2.0 * Uyz;
+        for (int a = 0; a < 3; a++) Ad[a] = fma(r, S[a], fma(2.0, D[a][a], c));
+        const double Xxy = (U[ip + jp + k] + U[im + jm + k]) - (U[im + jp + k] + U[ip + jm + k]);
+        const double Xxz = (U[ip + jo + kp] + U[im + jo + km]) - (U[im + jo + kp] + U[ip + jo + km]);
+        const double Xyz = (U[io + jp + kp] + U[io + jm + km]) - (U[io + jm + kp] + U[io + jp + km]);
+        Ao[0] = fma(r4, Xxy, D[0][1] + D[1][0]);
+        Ao[1] = fma(r4, Xxz, D[0][2] + D[2][0]);
+        Ao[2] = fma(r4, Xyz, D[1][2] + D[2][1]);
+        if (STORE)
 #pragma unroll
-        for (int a = 0; a < 3; a++) {
-            A[(int64_t)a * cnt + t] = Ad[a];
-            A[(int64_t)(3 + a) * cnt + t] = Ao[a];
-        }
-        AA[t] = (Ad[0] * Ad[0] + Ad[1] * Ad[1] + Ad[2] * Ad[2]) + 2.0 * (Ao[0] * Ao[0] + Ao[1] * Ao[1] + Ao[2] * Ao[2]);
+            for (int a = 0; a < 3; a++) {
+                A[(int64_t)a * cnt + t] = inv2h * Ad[a];
+                A[(int64_t)(3 + a) * cnt + t] = inv2h * Ao[a];
+            }
+        const double d = fma(Ad[0], Ad[0], fma(Ad[1], Ad[1], Ad[2] * Ad[2]));
+        const double o = fma(Ao[0], Ao[0], fma(Ao[1], Ao[1], Ao[2] * Ao[2]));
+        AA[t] = sc * fma(2.0, o, d);
     }
 }
 
+// A thread takes the cells k = 2q, 2q + 1 of a row: one 16-byte load per array,
+// one store to each colour's half-array.  sums: of s0 and its square.
 __global__ void __launch_bounds__(kBlock)
     k_psi_setup(int lgn, const double *__restrict__ psi, const double *__restrict__ s0, const double *__restrict__ AA,
-                double *__restrict__ u, double *__restrict__ c0, double *__restrict__ c1, double *__restrict__ f)
+                double *__restrict__ u, double *__restrict__ c0, double *__restrict__ c1, double *__restrict__ f,
+                const Sums sums)
 {
     pdl_begin();
-    const int64_t cnt = (int64_t)1 << (3 * lgn);
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt; t += (int64_t)gridDim.x * blockDim.x) {
-        int i, j, k;
-        scoord(lgn, t, i, j, k);
-        const int64_t id = nidx(lgn, i, j, k);
-        u[t] = psi[id] - 1.0;
-        c0[t] = s0[id];
-        c1[t] = AA[id];
-        f[t] = 0.0;
+    const int m = (1 << lgn) - 1;
+    const int64_t half = (int64_t)1 << (3 * lgn - 1);
+    double s = 0.0, q = 0.0;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < half; t += (int64_t)gridDim.x * blockDim.x) {
+        const int j = (int)(t >> (lgn - 1)) & m, i = (int)(t >> (2 * lgn - 1));
+        const int64_t even = ((i + j) & 1) ? half : 0, odd = half - even;  // colour of k = 2q, 2q + 1
+        const double2 p = reinterpret_cast<const double2 *>(psi)[t], a = reinterpret_cast<const double2 *>(s0)[t],
+                      b = reinterpret_cast<const double2 *>(AA)[t];
+        u[even + t] = p.x - 1.0;
+        u[odd + t] = p.y - 1.0;
+        c0[even + t] = a.x;
+        c0[odd + t] = a.y;
+        c1[even + t] = b.x;
+        c1[odd + t] = b.y;
+        f[even + t] = 0.0;
+        f[odd + t] = 0.0;
+        s += a.x + a.y;
+        q = fma(a.x, a.x, fma(a.y, a.y, q));
     }
+    block_sum2(s, q, sums);
 }
 
 // lapse equation for phi = alpha psi (Eq. sol-scheme-CMC with s = psi^-4 sigma),
@@ -338,13 +361,17 @@ void div_to_split(int n, double inv2h, const double *Fx, const double *Fy, const
 void aij_aa(int n, double inv2h, double ih2, const double *Vx, const double *Vy, const double *Vz, const double *U,
             double *A, double *AA, cudaStream_t st)
 {
-    GR_LAUNCH(k_aij_aa, grid_for((int64_t)n * n * n), kBlock, st, log2i(n), inv2h, ih2, Vx, Vy, Vz, U, A, AA);
+    const int g = grid_for((int64_t)n * n * n);
+    const double r = 2.0 * ih2 / inv2h;
+    if (A) GR_LAUNCH(k_aij_aa<true>, g, kBlock, st, log2i(n), inv2h, r, Vx, Vy, Vz, U, A, AA);
+    else GR_LAUNCH(k_aij_aa<false>, g, kBlock, st, log2i(n), inv2h, r, Vx, Vy, Vz, U, A, AA);
 }
 
 void psi_setup(int n, const double *psi, const double *s0, const double *AA, double *u, double *c0, double *c1,
-               double *f, cudaStream_t st)
+               double *f, const Sums &sums, cudaStream_t st)
 {
-    GR_LAUNCH(k_psi_setup, grid_for((int64_t)n * n * n), kBlock, st, log2i(n), psi, s0, AA, u, c0, c1, f);
+    GR_LAUNCH(k_psi_setup, wave_grid(k_psi_setup, (int64_t)n * n * n / 2), kBlock, st, log2i(n), psi, s0, AA, u, c0, c1,
+              f, sums);
 }
 
 void apsi_setup(int n, double h2, const double *psi, const double *apsi, const double *s0, const double *sig,

@@ -33,16 +33,6 @@ namespace {
 
 constexpr int kT64Ctas = 16, kT64Threads = 128;
 
-// 1/x by Newton's iteration r <- r + r (1 - x r) from the hardware's 20-bit
-// estimate: two steps leave about one unit in the last place
-__device__ __forceinline__ double recip64(double x)
-{
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
-}
-
 // arrays of levels 2^3 .. 16^3 (index 0 = 2^3); u and f of the top level in, u out
 struct T64Args {
     double *u;

@@ -97,7 +97,7 @@ struct gr_ctx {
     double *hscal = nullptr, *hscal_dev = nullptr;  // mapped pinned host scalars and their device alias
     double rho_dep = NAN;
     // what A6/AA hold for the V, U in the fields, and tmp (alpha psi psi^-7) for
-    // the psi, alpha psi in the fields: 0 nothing current, 1 FP64, 2 double-float pairs
+    // the psi, alpha psi in the fields: 0 nothing current, 1 FP64, 2 double-float pairs, 3 AA in FP64 alone
     int a_fmt = 0;
     int w_fmt = 0;
     bool tail_on = true;   // FP32 cycles: levels <= 16^3 in one block (GR_COARSE_TAIL=0 turns it off)
@@ -331,16 +331,19 @@ gr_status poisson_rhs_finish(gr_ctx *c, Level &F, double *ref)
     return GR_OK;
 }
 
-void ensure_aij(gr_ctx *c, const gr_fields *fl)
+// alone: the call forms one equation and reads AA only
+void ensure_aij(gr_ctx *c, const gr_fields *fl, bool alone = false)
 {
-    if (c->a_fmt == 1) return;
-    gr::aij_aa(c->n, 0.5 / c->h, 1.0 / (c->h * c->h), fl->V[0], fl->V[1], fl->V[2], fl->U, c->A6, c->AA, c->st);
-    c->a_fmt = 1;
+    if (c->a_fmt == 1 || (alone && c->a_fmt == 3)) return;
+    gr::aij_aa(c->n, 0.5 / c->h, 1.0 / (c->h * c->h), fl->V[0], fl->V[1], fl->V[2], fl->U, alone ? nullptr : c->A6, c->AA,
+               c->st);
+    c->a_fmt = alone ? 3 : 1;
 }
 
 // Build the fine-level unknown, right-hand side and coefficients of equation eq
 // (split layout) from the sources and current fields; fills info.
-gr_status setup_eq(gr_ctx *c, int eq, const gr_sources *s, const gr_fields *fl, double rho, double S_hat, EqInfo *info)
+gr_status setup_eq(gr_ctx *c, int eq, const gr_sources *s, const gr_fields *fl, double rho, double S_hat, EqInfo *info,
+                   bool alone = false)
 {
     const int n = c->n;
     const int64_t N = (int64_t)n * n * n;
@@ -363,14 +366,13 @@ gr_status setup_eq(gr_ctx *c, int eq, const gr_sources *s, const gr_fields *fl, 
         gr::div_to_split(n, 0.5 / c->h, Fv[0], Fv[1], Fv[2], -0.25, F.f, c->st);
         st = poisson_rhs_finish(c, F, &info->ref);
     } else if (eq == GR_PSI) {
-        ensure_aij(c, fl);
-        gr::psi_setup(n, fl->psi, s->s0, c->AA, F.u, F.c0, F.c1, F.f, c->st);
-        dsum(c, N, s->s0, true);
+        ensure_aij(c, fl, alone);
+        gr::psi_setup(n, fl->psi, s->s0, c->AA, F.u, F.c0, F.c1, F.f, sums_to(c, c->dscal, true), c->st);
         double a, q;
         st = read_scalars(c, &a, &q);
         info->ref = 2.0 * kPi * std::sqrt(q / N);
     } else if (eq == GR_APSI) {
-        ensure_aij(c, fl);
+        ensure_aij(c, fl, alone);
         gr::apsi_setup(n, c->h * c->h, fl->psi, fl->apsi, s->s0, s->sigma, c->AA, K2, Kdot, F.u, F.c0, F.c1, F.f,
                        c->tmp, c->st);
         c->w_fmt = 0;  // tmp now holds psi^5 Kdot
@@ -1711,7 +1713,7 @@ gr_status gr_residual(gr_ctx *c, gr_eq eq, const gr_sources *s, const gr_fields 
     c->a_fmt = 0;
     c->w_fmt = 0;
     EqInfo in;
-    st = setup_eq(c, eq, s, fl, rho, S_hat, &in);
+    st = setup_eq(c, eq, s, fl, rho, S_hat, &in, true);
     if (st != GR_OK) return st;
     double r;
     norm64(c, in.kind, rho, res_field);

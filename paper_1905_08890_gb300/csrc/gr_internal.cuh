@@ -150,6 +150,16 @@ struct Sums {
 };
 
 #ifdef __CUDACC__
+// 1/x by Newton's iteration r <- r + r (1 - x r) from the hardware's 20-bit
+// estimate: two steps leave about one unit in the last place
+__device__ __forceinline__ double recip64(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
 // the end of a reducing kernel, by every thread of the block, after thread 0
 // wrote the block's partials
 __device__ __forceinline__ void last_block_sum(const Sums &S)
@@ -446,12 +456,12 @@ void from_split(int n, const double *split, double *nat, double shift, const dou
 // f (split) = scale * div3(F) from natural F (3-point central differences).
 void div_to_split(int n, double inv2h, const double *Fx, const double *Fy, const double *Fz, double scale, double *f,
                   cudaStream_t st);
-// A_ij (6 natural arrays: xx yy zz xy xz yz) and AA (natural) from V, U.
+// A_ij (6 natural arrays: xx yy zz xy xz yz; A null: not stored) and AA (natural) from V, U.
 void aij_aa(int n, double inv2h, double ih2, const double *Vx, const double *Vy, const double *Vz, const double *U,
             double *A, double *AA, cudaStream_t st);
-// psi equation: u = psi - 1, c0 = s0, c1 = AA, f = 0 (split).
+// psi equation: u = psi - 1, c0 = s0, c1 = AA, f = 0 (split); sums of s0 and s0^2.
 void psi_setup(int n, const double *psi, const double *s0, const double *AA, double *u, double *c0, double *c1,
-               double *f, cudaStream_t st);
+               double *f, const Sums &sums, cudaStream_t st);
 // alpha psi equation: u = apsi - 1, c0 = m, c1 = 1/(6 + h^2 m), f = m - psi^5 Kdot (split);
 // g = psi^5 Kdot (natural scratch) for the reference norm.
 void apsi_setup(int n, double h2, const double *psi, const double *apsi, const double *s0, const double *sig,

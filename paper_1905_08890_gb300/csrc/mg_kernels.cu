@@ -59,6 +59,15 @@ __device__ __forceinline__ T nbsum(const T *__restrict__ u, int lgn, int i, int 
            u[sidx(lgn, i, (j - 1) & m, k)] + u[sidx(lgn, i, j, (k + 1) & m)] + u[sidx(lgn, i, j, (k - 1) & m)];
 }
 
+// the psi operator added to lap (the Laplacian, or it less a right-hand side):
+// iv (2 pi s0 + AA/8 iv^6) and one Newton reciprocal, since FP64 issue is the cost
+__device__ __forceinline__ double psi_resid(double lap, double uc, double s0, double aa, double rho)
+{
+    const double v = 1.0 + uc, iv = recip64(v), iv2 = iv * iv, v2 = v * v;
+    const double q = fma(0.125 * aa, iv2 * iv2 * iv2, 2.0 * kPi * s0);
+    return fma(-2.0 * kPi * rho, v2 * v2 * v, fma(q, iv, lap));
+}
+
 // L(u) at one cell: u value uc, neighbour sum nb, coefficients at the cell
 template <typename T, int KIND>
 __device__ __forceinline__ T op_cell(T uc, T nb, T ih2, T c0, T c1, T rho)
@@ -66,10 +75,7 @@ __device__ __forceinline__ T op_cell(T uc, T nb, T ih2, T c0, T c1, T rho)
     T lap = (nb - T(6) * uc) * ih2;
     if (KIND == KPOISSON) return lap;
     if (KIND == KHELM) return lap - c0 * uc;
-    const double v = 1.0 + (double)uc, iv = 1.0 / v, iv2 = iv * iv, iv4 = iv2 * iv2;
-    const double v2 = v * v, v4 = v2 * v2;
-    return (T)((double)lap + 2.0 * kPi * (double)c0 * iv + 0.125 * (double)c1 * (iv4 * iv2 * iv) -
-               2.0 * kPi * (double)rho * (v4 * v));
+    return (T)psi_resid((double)lap, (double)uc, (double)c0, (double)c1, (double)rho);
 }
 
 template <typename T, int KIND>
@@ -79,6 +85,9 @@ __device__ __forceinline__ T resid_cell(const T *__restrict__ u, const T *__rest
     const int64_t id = sidx(lgn, i, j, k);
     const T a0 = (KIND == KPOISSON) ? T(0) : c0[id];
     const T a1 = (KIND == KPSI) ? c1[id] : T(0);
+    if (KIND == KPSI)
+        return (T)psi_resid(fma((double)nbsum(u, lgn, i, j, k) - 6.0 * (double)u[id], (double)ih2, -(double)f[id]),
+                            (double)u[id], (double)a0, (double)a1, (double)rho);
     return op_cell<T, KIND>(u[id], nbsum(u, lgn, i, j, k), ih2, a0, a1, rho) - f[id];
 }
 
@@ -115,13 +124,13 @@ __global__ void __launch_bounds__(kBlock)
             own[t] = (nb - h2 * f[c]) * c1[c];  // c1 = 1/(6 + h^2 m)
         } else {
             const double uc = (double)own[t];
-            const double v = 1.0 + uc, iv = 1.0 / v, iv2 = iv * iv, iv4 = iv2 * iv2, iv8 = iv4 * iv4;
+            const double v = 1.0 + uc, iv = recip64(v), iv2 = iv * iv, iv6 = iv2 * iv2 * iv2;
             const double v2 = v * v, v4 = v2 * v2;
-            const double s0 = (double)c0[c], aa = (double)c1[c], ihd = (double)ih2, rh = (double)rho;
-            const double g = ((double)nb - 6.0 * uc) * ihd + 2.0 * kPi * s0 * iv + 0.125 * aa * (iv4 * iv2 * iv) -
-                             2.0 * kPi * rh * (v4 * v) - (double)f[c];
-            const double dg = -6.0 * ihd - 2.0 * kPi * s0 * iv2 - 0.875 * aa * iv8 - 10.0 * kPi * rh * v4;
-            own[t] = (T)(uc - g / dg);
+            const double sp = 2.0 * kPi * (double)c0[c], aa = 0.125 * (double)c1[c], ihd = (double)ih2,
+                         rp = 2.0 * kPi * (double)rho;
+            const double g = fma(-rp, v4 * v, fma(fma(aa, iv6, sp), iv, fma(fma(-6.0, uc, (double)nb), ihd, -(double)f[c])));
+            const double dg = fma(-5.0 * rp, v4, fma(-fma(7.0 * aa, iv6, sp), iv2, -6.0 * ihd));
+            own[t] = (T)fma(-g, recip64(dg), uc);
         }
     }
 }
@@ -758,7 +767,7 @@ __global__ void __launch_bounds__(kBlock)
         scoord(lgn, t, i, j, k);
         const double e = (double)resid_cell<T, KIND>(u, f, c0, c1, lgn, i, j, k, ih2, rho);
         s2 += e * e;
-        su += (double)u[t];
+        if (KIND == KPOISSON) su += (double)u[t];  // read for the zero mean of the Poisson-type solutions
         if (eps_nat) eps_nat[((((int64_t)i << lgn) + j) << lgn) + k] = e;
     }
     block_sum2(s2, su, sums);
@@ -783,7 +792,7 @@ __global__ void __launch_bounds__(kBlock)
         su += u[t];
         r32[t] = (float)(-e);
         if (KIND == KPSI) {
-            const double v = 1.0 + u[t], iv = 1.0 / v, iv2 = iv * iv, iv4 = iv2 * iv2, v2 = v * v;
+            const double v = 1.0 + u[t], iv = recip64(v), iv2 = iv * iv, iv4 = iv2 * iv2, v2 = v * v;
             const double mj = 2.0 * kPi * c0[t] * iv2 + 0.875 * c1[t] * (iv4 * iv4) + 10.0 * kPi * rho * (v2 * v2);
             const float mf = (float)mj;
             m32[t] = mf;
