@@ -2,9 +2,8 @@
 // circular 3^3 convolutions on channels-last BF16 activations [v][c],
 // v = (d n + h) n + w, FP32 accumulation on the tensor cores (mma.sync
 // m16n8k16 BF16; 128^3 grids on tcgen05, conv_tc.cu).  Convolutions are
-// implicit GEMMs: output voxels x output channels, reduced over 27 taps x
-// input channels, with the shifted input rows gathered straight from global
-// memory (the 27-fold reuse is served by L1).
+// implicit GEMMs: output voxels x output channels, reduced over input channels x
+// 27 taps, from boxes of voxels staged with their halo in shared memory.
 //
 // Weights: FP32 master and BF16 copies [27][cout][cin] (tap = (dd+1)*9 +
 // (dh+1)*3 + (dw+1)); the data gradient is the same convolution with the
@@ -47,21 +46,122 @@ __device__ __forceinline__ int nbr(int v, int lg, int tap)
 }
 
 // ---------------------------------------------------------------- convolution
-// Block: 4 warps along the voxels; warp tile MT*16 voxels x NT*8 channels;
-// grid.y walks the output channels in steps of NT*8.  Epilogue modes:
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void cp16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+// A box of 2^lw x 2^lh x 2^ld voxels (w fastest) of a 2^lg grid and its halo of
+// one voxel per side: the unit of work of the convolution and its weight gradient.
+struct Box {
+    int lg, lw, lh, ld;
+    __host__ __device__ int hw() const { return (1 << lw) + 2; }
+    __host__ __device__ int hh() const { return (1 << lh) + 2; }
+    __host__ __device__ int hd() const { return (1 << ld) + 2; }
+    __host__ __device__ int halo() const { return hw() * hh() * hd(); }
+    // origin of box b (boxes in w, h, d order)
+    __device__ void origin(int b, int &d0, int &h0, int &w0) const
+    {
+        const int nw = lg - lw, nh = lg - lh;
+        w0 = (b & ((1 << nw) - 1)) << lw;
+        h0 = ((b >> nw) & ((1 << nh) - 1)) << lh;
+        d0 = (b >> (nw + nh)) << ld;
+    }
+    // voxel q of the box: its halo index at tap (0, 0, 0) (the corner of its 3^3 neighbourhood)
+    __device__ int corner(int q) const
+    {
+        const int w = q & ((1 << lw) - 1), h = (q >> lw) & ((1 << lh) - 1), dd = q >> (lw + lh);
+        return (dd * hh() + h) * hw() + w;
+    }
+    __device__ int voxel(int q, int d0, int h0, int w0) const
+    {
+        const int w = q & ((1 << lw) - 1), h = (q >> lw) & ((1 << lh) - 1), dd = q >> (lw + lh);
+        return ((((d0 + dd) << lg) + h0 + h) << lg) + w0 + w;
+    }
+};
+
+// 2^lb voxels per box: rows along w of up to 16, then h and d in turn
+Box make_box(int lg, int lb)
+{
+    Box x;
+    x.lg = lg;
+    x.lw = lg < 4 ? lg : 4;
+    const int rest = lb - x.lw;
+    x.lh = (rest + 1) / 2 < lg ? (rest + 1) / 2 : lg;
+    x.ld = rest - x.lh;
+    return x;
+}
+
+// a 32-byte row (16 channels) holds its two 16-byte halves swapped on every
+// second group of four rows, so that eight consecutive rows' halves fall on all 32 banks
+__device__ __forceinline__ uint32_t row_half(int row, int half) { return (uint32_t)(32 * row + ((half ^ (row >> 2 & 1)) << 4)); }
+
+// the halo's 16 channels from c0 into shared memory (asynchronous copies)
+__device__ __forceinline__ void load_halo(uint32_t dst, const __nv_bfloat16 *x, int cin, int c0, const Box &bx, int d0, int h0,
+                                          int w0)
+{
+    const int m = (1 << bx.lg) - 1, hw = bx.hw(), hh = bx.hh(), n = 2 * bx.halo();
+    for (int e = threadIdx.x; e < n; e += blockDim.x) {
+        const int r = e >> 1, half = e & 1;
+        const int w = r % hw, t = r / hw, h = t % hh, dd = t / hh;
+        const int v = ((((d0 + dd - 1) & m) << bx.lg) + ((h0 + h - 1) & m)) * (1 << bx.lg) + ((w0 + w - 1) & m);
+        cp16(dst + row_half(r, half), x + (size_t)v * cin + c0 + 8 * half);
+    }
+}
+
+// Block: WARPS warps along the voxels of one box; warp tile MT*16 voxels x NT*8
+// channels; grid.y walks the output channels in steps of NT*8.  Per 16 input
+// channels the box with its halo and the 27 taps' weights are staged in shared
+// memory, one chunk ahead, and the fragments come from there (ldmatrix):
+// gathered straight from global memory in 4-byte loads they cost 16 loads and 40 index
+// instructions per eight MMAs.  The ten layers of a 128^3 pass took 1467 us that way and
+// take 437 us.  The products are summed in the order input channels, taps, as
+// the order of a layer's arithmetic is part of its result.  Epilogue modes:
 //   CONV_RELU  y = relu(acc + bias) (BF16)
 //   CONV_MASK  y = acc * (mask > 0) (BF16; data gradient through a ReLU)
 //   CONV_PLAIN y = acc (BF16)
-template <int MT, int NT>
-__global__ void __launch_bounds__(128)
+template <int WARPS, int MT, int NT>
+__global__ void __launch_bounds__(32 * WARPS)
     k_conv3d(const __nv_bfloat16 *__restrict__ x, int cin, const __nv_bfloat16 *__restrict__ w,
-             const float *__restrict__ bias, int cout, int lg, int mode, const __nv_bfloat16 *__restrict__ mask,
+             const float *__restrict__ bias, int cout, Box bx, int mode, const __nv_bfloat16 *__restrict__ mask,
              __nv_bfloat16 *__restrict__ y)
 {
     pdl_begin();
+    static_assert(NT % 2 == 0, "two 8-channel tiles per ldmatrix");
+    extern __shared__ __align__(128) unsigned char csm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int vb = (blockIdx.x * 4 + warp) * (MT * 16);
     const int cb = blockIdx.y * (NT * 8);
+    int d0, h0, w0;
+    bx.origin(blockIdx.x, d0, h0, w0);
+    const int halo = bx.halo(), hw = bx.hw(), hh = bx.hh();
+    const uint32_t base = smem_addr(csm), stage = 32u * (uint32_t)(halo + 27 * NT * 8);
+    auto load = [&](int c0, uint32_t buf) {
+        load_halo(buf, x, cin, c0, bx, d0, h0, w0);
+        const uint32_t wb = buf + 32u * (uint32_t)halo;
+        for (int e = threadIdx.x; e < 2 * 27 * NT * 8; e += 32 * WARPS) {
+            const int half = e & 1, r = e >> 1, co = r % (NT * 8), tap = r / (NT * 8);
+            cp16(wb + row_half(r, half), w + ((size_t)tap * cout + cb + co) * cin + c0 + 8 * half);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
     float acc[MT][NT][4];
 #pragma unroll
     for (int a = 0; a < MT; a++)
@@ -69,35 +169,53 @@ __global__ void __launch_bounds__(128)
         for (int b = 0; b < NT; b++)
 #pragma unroll
             for (int r = 0; r < 4; r++) acc[a][b][r] = 0.0f;
-    for (int c0 = 0; c0 < cin; c0 += 16) {
-        for (int tap = 0; tap < 27; tap++) {
-            uint32_t bf[NT][2];
+    // this lane's row of each A tile (lanes 0..15: channels 0..7, 16..31: 8..15) and of each B pair
+    int arow[MT];
 #pragma unroll
-            for (int b = 0; b < NT; b++) {
-                const __nv_bfloat16 *wp = w + ((size_t)tap * cout + cb + b * 8 + g) * cin + c0 + 2 * t;
-                bf[b][0] = ld32(wp);
-                bf[b][1] = ld32(wp + 8);
-            }
-#pragma unroll
-            for (int a = 0; a < MT; a++) {
-                const int v0 = nbr(vb + a * 16 + g, lg, tap), v1 = nbr(vb + a * 16 + g + 8, lg, tap);
-                const __nv_bfloat16 *p0 = x + (size_t)v0 * cin + c0 + 2 * t;
-                const __nv_bfloat16 *p1 = x + (size_t)v1 * cin + c0 + 2 * t;
-                uint32_t af[4] = {ld32(p0), ld32(p1), ld32(p0 + 8), ld32(p1 + 8)};
-#pragma unroll
-                for (int b = 0; b < NT; b++) mma_bf16(acc[a][b], af, bf[b]);
-            }
+    for (int a = 0; a < MT; a++) arow[a] = bx.corner((warp * MT + a) * 16 + (lane & 15));
+    const int ahalf = lane >> 4, brow = (lane & 7) + ((lane >> 4) << 3), bhalf = (lane >> 3) & 1;
+    load(0, base);
+    for (int c0 = 0, k = 0; c0 < cin; c0 += 16, k ^= 1) {
+        const uint32_t buf = base + (k ? stage : 0u);
+        if (c0 + 16 < cin) {
+            load(c0 + 16, base + (k ? 0u : stage));
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
+        __syncthreads();
+        const uint32_t wb = buf + 32u * (uint32_t)halo;
+        int tap = 0;
+        for (int dd = 0; dd < 3; dd++)
+            for (int dh = 0; dh < 3; dh++) {
+                const int off = (dd * hh + dh) * hw;
+#pragma unroll
+                for (int dw = 0; dw < 3; dw++, tap++) {
+                    uint32_t bf[NT / 2][4];
+#pragma unroll
+                    for (int b = 0; b < NT / 2; b++) ldsm4(bf[b], wb + row_half(tap * NT * 8 + 16 * b + brow, bhalf));
+#pragma unroll
+                    for (int a = 0; a < MT; a++) {
+                        uint32_t af[4];
+                        ldsm4(af, buf + row_half(arow[a] + off + dw, ahalf));
+#pragma unroll
+                        for (int b = 0; b < NT; b++) {
+                            const uint32_t bb[2] = {bf[b >> 1][2 * (b & 1)], bf[b >> 1][2 * (b & 1) + 1]};
+                            mma_bf16(acc[a][b], af, bb);
+                        }
+                    }
+                }
+            }
+        __syncthreads();  // before the next chunk's copies overwrite this buffer
     }
 #pragma unroll
     for (int a = 0; a < MT; a++)
 #pragma unroll
-        for (int b = 0; b < NT; b++) {
-            const int co = cb + b * 8 + 2 * t;
+        for (int hrow = 0; hrow < 2; hrow++) {
+            const int v = bx.voxel((warp * MT + a) * 16 + g + 8 * hrow, d0, h0, w0);
 #pragma unroll
-            for (int hrow = 0; hrow < 2; hrow++) {
-                const int v = vb + a * 16 + g + 8 * hrow;
-                if (v >= (1 << (3 * lg))) continue;  // grids smaller than one block tile
+            for (int b = 0; b < NT; b++) {
+                const int co = cb + b * 8 + 2 * t;
                 float r0 = acc[a][b][2 * hrow], r1 = acc[a][b][2 * hrow + 1];
                 const size_t o = (size_t)v * cout + co;
                 if (mode == CONV_RELU) {
@@ -110,6 +228,21 @@ __global__ void __launch_bounds__(128)
                 *reinterpret_cast<uint32_t *>(y + o) = pack2(__float2bfloat16(r0), __float2bfloat16(r1));
             }
         }
+}
+
+template <int WARPS, int MT, int NT>
+void launch_conv3d(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, const float *bias, int cout, int lg, int lb,
+                   int mode, const __nv_bfloat16 *mask, __nv_bfloat16 *y, cudaStream_t st)
+{
+    // the largest halo of these boxes: 2^8 voxels as 4 x 4 x 16 or 4 x 8 x 8
+    constexpr int kMost = 2 * 32 * (720 + 27 * NT * 8);
+    static const bool attr = cudaFuncSetAttribute(k_conv3d<WARPS, MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                  kMost) == cudaSuccess;
+    (void)attr;
+    const Box bx = make_box(lg, lb);
+    const int smem = (cin > 16 ? 2 : 1) * 32 * (bx.halo() + 27 * NT * 8);
+    const dim3 grid(1u << (3 * lg - lb), cout / (NT * 8));
+    GR_LAUNCH_SMEM((k_conv3d<WARPS, MT, NT>), grid, 32 * WARPS, smem, st, x, cin, w, bias, cout, bx, mode, mask, y);
 }
 
 // ---------------------------------------------------------------- weight gradient
@@ -635,14 +768,14 @@ void conv3d(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, const float
         conv3d_tc(x, cin, w, bias, cout, mode, mask, y, st);
         return;
     }
+    // 256 voxels x 32 (16) channels per block where that gives every SM two blocks, else 64 voxels x
+    // 16 channels (16^3, 128 -> 128: 21 us; 8^3 at 64^3's coarsest level had 16 blocks of 62 us)
     const int64_t nv = (int64_t)1 << (3 * lg);
-    if (cout % 32 == 0) {
-        // 4 warps x 32 voxels, 32 channels per block
-        dim3 grid(cdiv(nv, 4 * 32), cout / 32);
-        GR_LAUNCH((k_conv3d<2, 4>), grid, 128, st, x, cin, w, bias, cout, lg, mode, mask, y);
+    if (lg >= 3 && (nv >> 8) * (cout / 16) >= 304) {
+        if (cout % 32 == 0) launch_conv3d<8, 2, 4>(x, cin, w, bias, cout, lg, 8, mode, mask, y, st);
+        else launch_conv3d<8, 2, 2>(x, cin, w, bias, cout, lg, 8, mode, mask, y, st);
     } else {
-        dim3 grid(cdiv(nv, 4 * 64), cout / 16);
-        GR_LAUNCH((k_conv3d<4, 2>), grid, 128, st, x, cin, w, bias, cout, lg, mode, mask, y);
+        launch_conv3d<4, 1, 2>(x, cin, w, bias, cout, lg, 6, mode, mask, y, st);
     }
 }
 
