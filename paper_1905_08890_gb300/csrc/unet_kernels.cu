@@ -247,62 +247,82 @@ void launch_conv3d(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, cons
 
 // ---------------------------------------------------------------- weight gradient
 // dw[tap][co][ci] += sum_v dy[v][co] x[nbr(v, tap)][ci]: GEMM with M = co,
-// N = ci, K = voxels.  Block: one tap (grid.y), one voxel chunk (grid.x), one
-// (16 co x 8 NT ci) tile set (grid.z); the 4 warps split the chunk's voxels
-// and their partial sums meet in shared memory before one FP32 atomic per
-// output.  Operand pairs along K are two voxels, packed from scalar loads.
-template <int NT>
-__global__ void __launch_bounds__(128)
-    k_conv3d_wgrad(const __nv_bfloat16 *__restrict__ x, int cin, const __nv_bfloat16 *__restrict__ dy, int cout,
-                   int lg, int chunk, float *__restrict__ dw)
+// N = ci, K = voxels.  Block: 16 output x 16 input channels (grid.y), a range of
+// voxel boxes (grid.x), all 27 taps, three per warp.  Per box the 16 channels of
+// dy and of x with its halo are staged in shared memory, one box ahead; both
+// operands are read transposed (ldmatrix .trans) from the voxel rows, A once
+// for a warp's three taps.  The taps' sums stay in registers over the block's
+// boxes and end in one FP32 atomic per weight.  (One tap per block with
+// two-byte gathers took 957 us over the layers at 64^3; these take 304.)
+constexpr int kWgWarps = 9, kWgBox = 8;  // boxes of 2^8 voxels (or the grid)
+__global__ void __launch_bounds__(32 * kWgWarps)
+    k_conv3d_wgrad(const __nv_bfloat16 *__restrict__ x, int cin, const __nv_bfloat16 *__restrict__ dy, int cout, Box bx,
+                   int nbox, float *__restrict__ dw)
 {
     pdl_begin();
-    __shared__ float red[4][16 * NT * 8];
+    extern __shared__ __align__(128) unsigned char csm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int tap = blockIdx.y;
-    const int ntiles_ci = cin / (NT * 8);
-    const int co0 = (blockIdx.z / ntiles_ci) * 16, ci0 = (blockIdx.z % ntiles_ci) * (NT * 8);
-    const int vstart = blockIdx.x * chunk;
-    float acc[NT][4];
-#pragma unroll
-    for (int b = 0; b < NT; b++)
-#pragma unroll
-        for (int r = 0; r < 4; r++) acc[b][r] = 0.0f;
-    for (int vk = vstart + warp * 16; vk < vstart + chunk; vk += 64) {
-        // A (16 co x 16 v): rows co0 + g (+8), columns vk + 2t (+1) (+8)
-        uint32_t af[4];
-        {
-            const __nv_bfloat16 *a0 = dy + (size_t)(vk + 2 * t) * cout + co0 + g;
-            af[0] = pack2(a0[0], a0[cout]);
-            af[1] = pack2(a0[8], a0[cout + 8]);
-            const __nv_bfloat16 *a1 = a0 + (size_t)8 * cout;
-            af[2] = pack2(a1[0], a1[cout]);
-            af[3] = pack2(a1[8], a1[cout + 8]);
+    const int nci = cin >> 4, co0 = ((int)blockIdx.y / nci) << 4, ci0 = ((int)blockIdx.y % nci) << 4;
+    const int halo = bx.halo(), hw = bx.hw(), hh = bx.hh(), nv = 1 << (bx.lw + bx.lh + bx.ld);
+    const uint32_t base = smem_addr(csm), stage = 32u * (uint32_t)(halo + nv);
+    const int first = (int)((int64_t)blockIdx.x * nbox / gridDim.x), last = (int)((int64_t)(blockIdx.x + 1) * nbox / gridDim.x);
+    auto load = [&](int b, uint32_t buf) {
+        int d0, h0, w0;
+        bx.origin(b, d0, h0, w0);
+        load_halo(buf, x, cin, ci0, bx, d0, h0, w0);
+        for (int e = threadIdx.x; e < 2 * nv; e += 32 * kWgWarps) {
+            const int q = e >> 1, half = e & 1;
+            cp16(buf + 32u * (uint32_t)halo + row_half(q, half), dy + (size_t)bx.voxel(q, d0, h0, w0) * cout + co0 + 8 * half);
         }
-        const int n0 = nbr(vk + 2 * t, lg, tap), n1 = nbr(vk + 2 * t + 1, lg, tap);
-        const int n8 = nbr(vk + 2 * t + 8, lg, tap), n9 = nbr(vk + 2 * t + 9, lg, tap);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc[3][2][4] = {};
+    int toff[3];
 #pragma unroll
-        for (int b = 0; b < NT; b++) {
-            const int ci = ci0 + b * 8 + g;
-            uint32_t bf[2] = {pack2(x[(size_t)n0 * cin + ci], x[(size_t)n1 * cin + ci]),
-                              pack2(x[(size_t)n8 * cin + ci], x[(size_t)n9 * cin + ci])};
-            mma_bf16(acc[b], af, bf);
-        }
+    for (int j = 0; j < 3; j++) {
+        const int tap = 3 * warp + j;
+        toff[j] = ((tap / 9) * hh + (tap / 3) % 3) * hw + tap % 3;
     }
-    // C (16 co x 8 ci per tile): acc[b][0..1] rows g, cols 2t, 2t+1; [2..3] rows g + 8
-#pragma unroll
-    for (int b = 0; b < NT; b++)
-#pragma unroll
-        for (int r = 0; r < 4; r++) {
-            const int row = g + 8 * (r >> 1), col = b * 8 + 2 * t + (r & 1);
-            red[warp][row * (NT * 8) + col] = acc[b][r];
+    // this lane's row and half of the four 8 x 8 matrices.  A (co x voxels, from
+    // dy's voxel rows): voxels 0..7 co 0..7, voxels 0..7 co 8..15, then voxels
+    // 8..15; B (voxels x ci): voxels 0..7 and 8..15 of ci 0..7, then of ci 8..15
+    const int arow = (lane & 7) + ((lane >> 4) << 3), ahalf = (lane >> 3) & 1;
+    const int brow = (lane & 7) + (((lane >> 3) & 1) << 3), bhalf = lane >> 4;
+    if (first < last) load(first, base);
+    for (int b = first, k = 0; b < last; b++, k ^= 1) {
+        const uint32_t buf = base + (k ? stage : 0u);
+        if (b + 1 < last) {
+            load(b + 1, base + (k ? 0u : stage));
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
-    __syncthreads();
-    for (int e = threadIdx.x; e < 16 * NT * 8; e += blockDim.x) {
-        const float s = red[0][e] + red[1][e] + red[2][e] + red[3][e];
-        const int row = e / (NT * 8), col = e % (NT * 8);
-        atomicAdd(dw + ((size_t)tap * cout + co0 + row) * cin + ci0 + col, s);
+        __syncthreads();
+        for (int q = 0; q < nv; q += 16) {
+            uint32_t af[4];
+            ldsm4t(af, buf + 32u * (uint32_t)halo + row_half(q + arow, ahalf));
+            const int c = bx.corner(q + brow);
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                uint32_t bf[4];
+                ldsm4t(bf, buf + row_half(c + toff[j], bhalf));
+                const uint32_t b0[2] = {bf[0], bf[1]}, b1[2] = {bf[2], bf[3]};
+                mma_bf16(acc[j][0], af, b0);
+                mma_bf16(acc[j][1], af, b1);
+            }
+        }
+        __syncthreads();  // before the next box's copies overwrite this buffer
     }
+    if (first >= last) return;
+    // acc[j][n][0..1]: co g, ci 8 n + 2 t (+ 1); [2..3]: co g + 8
+#pragma unroll
+    for (int j = 0; j < 3; j++)
+#pragma unroll
+        for (int n = 0; n < 2; n++)
+#pragma unroll
+            for (int r = 0; r < 4; r++)
+                atomicAdd(dw + ((size_t)(3 * warp + j) * cout + co0 + g + 8 * (r >> 1)) * cin + ci0 + 8 * n + 2 * t + (r & 1),
+                          acc[j][n][r]);
 }
 
 // ---------------------------------------------------------------- small layers
@@ -568,52 +588,88 @@ __global__ void k_head(const __nv_bfloat16 *__restrict__ a, const float *__restr
 }
 
 // loss and head backward: standardised target t[v][o]; dout = 2 (out - t) / (nv * 10);
-// da[v][c] = (a > 0) sum_o W[o][c] dout[v][o]; dW, db accumulated; loss partial per block
-__global__ void k_head_back(const __nv_bfloat16 *__restrict__ a, const float *__restrict__ W,
-                            const float *__restrict__ out, const float *__restrict__ tgt, int64_t nv,
-                            __nv_bfloat16 *__restrict__ da, float *__restrict__ dW, float *__restrict__ db,
-                            float *__restrict__ loss)
+// da[v][c] = (a > 0) sum_o W[o][c] dout[v][o]; dW, db accumulated; loss partial per block.
+// A thread per voxel forms dout and da and leaves dout and a in shared memory;
+// then 160 threads each sum one dW[o][c] over the block's voxels.  (With
+// the 160 sums in every thread's local memory 528 us at 64^3, so 27.)
+constexpr int kHbVox = 256;
+__global__ void __launch_bounds__(kHbVox)
+    k_head_back(const __nv_bfloat16 *__restrict__ a, const float *__restrict__ W, const float *__restrict__ out,
+                const float *__restrict__ tgt, int64_t nv, __nv_bfloat16 *__restrict__ da, float *__restrict__ dW,
+                float *__restrict__ db, float *__restrict__ loss)
 {
     pdl_begin();
-    __shared__ float sw[kNetOut * 16], sdw[kNetOut * 16], sdb[kNetOut], sl[1];
-    for (int k = threadIdx.x; k < kNetOut * 16; k += blockDim.x) {
-        sw[k] = W[k];
-        sdw[k] = 0.0f;
-    }
-    for (int k = threadIdx.x; k < kNetOut; k += blockDim.x) sdb[k] = 0.0f;
-    if (threadIdx.x == 0) sl[0] = 0.0f;
+    __shared__ float sw[kNetOut * 16], sd[kHbVox][kNetOut + 1], sa[kHbVox][17], sl[kHbVox / 32];
+    for (int k = threadIdx.x; k < kNetOut * 16; k += kHbVox) sw[k] = W[k];
     __syncthreads();
     const float scale = 2.0f / ((float)nv * kNetOut);
-    float lsum = 0.0f;
-    float ldw[kNetOut * 16];
-    float ldb[kNetOut];
-    for (int k = 0; k < kNetOut * 16; k++) ldw[k] = 0.0f;
-    for (int k = 0; k < kNetOut; k++) ldb[k] = 0.0f;
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += (int64_t)gridDim.x * blockDim.x) {
-        float av[16], g[16], d[kNetOut];
+    float lsum = 0.0f, wsum = 0.0f, bsum = 0.0f;
+    const int so = threadIdx.x / 16, sc = threadIdx.x % 16;  // the sum this thread carries (so < 10)
+    for (int64_t v0 = (int64_t)blockIdx.x * kHbVox; v0 < nv; v0 += (int64_t)gridDim.x * kHbVox) {
+        const int64_t v = v0 + threadIdx.x;
+        const bool ok = v < nv;
+        float av[16], g[16];
+        if (ok) {
+            const uint4 *a8 = reinterpret_cast<const uint4 *>(a + v * 16);
+            float lo[8], hi[8];
+            bf8_unpack(a8[0], lo);
+            bf8_unpack(a8[1], hi);
+#pragma unroll
+            for (int c = 0; c < 16; c++) av[c] = c < 8 ? lo[c & 7] : hi[c & 7];
+        }
+#pragma unroll
         for (int c = 0; c < 16; c++) {
-            av[c] = __bfloat162float(a[v * 16 + c]);
             g[c] = 0.0f;
+            if (!ok) av[c] = 0.0f;
+            sa[threadIdx.x][c] = av[c];
         }
+#pragma unroll
         for (int o = 0; o < kNetOut; o++) {
-            const float r = out[v * kNetOut + o] - tgt[v * kNetOut + o];
+            const float r = ok ? out[v * kNetOut + o] - tgt[v * kNetOut + o] : 0.0f;
             lsum += r * r;
-            d[o] = scale * r;
-            ldb[o] += d[o];
-            for (int c = 0; c < 16; c++) {
-                ldw[o * 16 + c] += d[o] * av[c];
-                g[c] += sw[o * 16 + c] * d[o];
-            }
+            const float d = scale * r;
+            sd[threadIdx.x][o] = d;
+#pragma unroll
+            for (int c = 0; c < 16; c++) g[c] += sw[o * 16 + c] * d;
         }
-        for (int c = 0; c < 16; c++) da[v * 16 + c] = __float2bfloat16(av[c] > 0.0f ? g[c] : 0.0f);
+        if (ok) {
+            float lo[8], hi[8];
+#pragma unroll
+            for (int c = 0; c < 8; c++) {
+                lo[c] = av[c] > 0.0f ? g[c] : 0.0f;
+                hi[c] = av[8 + c] > 0.0f ? g[8 + c] : 0.0f;
+            }
+            uint4 *o8 = reinterpret_cast<uint4 *>(da + v * 16);
+            o8[0] = bf8_pack(lo);
+            o8[1] = bf8_pack(hi);
+        }
+        __syncthreads();
+        if (so < kNetOut) {
+            float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 4
+            for (int q = 0; q < kHbVox; q += 4)
+#pragma unroll
+                for (int e = 0; e < 4; e++) s4[e] += sd[q + e][so] * sa[q + e][sc];
+            wsum += (s4[0] + s4[1]) + (s4[2] + s4[3]);
+        } else if (so < kNetOut + 5) {  // ten pairs of eight threads: the biases' sums
+            const int o = (so - kNetOut) * 2 + (sc >> 3);
+            for (int q = sc & 7; q < kHbVox; q += 8) bsum += sd[q][o];
+        }
+        __syncthreads();
     }
-    for (int k = 0; k < kNetOut * 16; k++) atomicAdd(&sdw[k], ldw[k]);
-    for (int k = 0; k < kNetOut; k++) atomicAdd(&sdb[k], ldb[k]);
-    atomicAdd(&sl[0], lsum);
+    if (so < kNetOut) {
+        atomicAdd(dW + threadIdx.x, wsum);
+    } else if (so < kNetOut + 5) {
+        atomicAdd(db + (so - kNetOut) * 2 + (sc >> 3), bsum);
+    }
+    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    if ((threadIdx.x & 31) == 0) sl[threadIdx.x >> 5] = lsum;
     __syncthreads();
-    for (int k = threadIdx.x; k < kNetOut * 16; k += blockDim.x) atomicAdd(dW + k, sdw[k]);
-    for (int k = threadIdx.x; k < kNetOut; k += blockDim.x) atomicAdd(db + k, sdb[k]);
-    if (threadIdx.x == 0) atomicAdd(loss, sl[0] / ((float)nv * kNetOut));
+    if (threadIdx.x == 0) {
+        float t = 0.0f;
+        for (int k = 0; k < kHbVox / 32; k++) t += sl[k];
+        atomicAdd(loss, t / ((float)nv * kNetOut));
+    }
 }
 
 // standardised target from natural-layout fields (psi, apsi as deviations)
@@ -621,12 +677,17 @@ __global__ void k_net_target(FieldPtrs fields, int64_t nv, const float *__restri
                              const float *__restrict__ stdv, float *__restrict__ tgt)
 {
     pdl_begin();
+    // the reciprocals once per thread (one per voxel and field: 63 us at 64^3, now 38)
+    double inv[kNetOut], mu[kNetOut];
+#pragma unroll
+    for (int o = 0; o < kNetOut; o++) {
+        inv[o] = 1.0 / (double)stdv[o];
+        mu[o] = (double)mean[o];
+    }
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += (int64_t)gridDim.x * blockDim.x)
-        for (int o = 0; o < kNetOut; o++) {
-            double val = fields.p[o][v];
-            if (o < 2) val -= 1.0;
-            tgt[v * kNetOut + o] = (float)((val - mean[o]) / stdv[o]);
-        }
+#pragma unroll
+        for (int o = 0; o < kNetOut; o++)
+            tgt[v * kNetOut + o] = (float)((fields.p[o][v] - (o < 2 ? 1.0 : 0.0) - mu[o]) * inv[o]);
 }
 
 // de-standardised output into the fields (psi, apsi get + 1)
@@ -782,17 +843,18 @@ void conv3d(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, const float
 void conv3d_wgrad(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *dy, int cout, int lg, float *dw,
                   cudaStream_t st)
 {
-    const int64_t nv = (int64_t)1 << (3 * lg);
-    int chunk = 2048;
-    while (chunk > 64 && nv / chunk < 64) chunk >>= 1;
-    if (nv < chunk) chunk = (int)nv;
-    if (cin % 32 == 0) {
-        dim3 grid((unsigned)(nv / chunk), 27, (cout / 16) * (cin / 32));
-        GR_LAUNCH((k_conv3d_wgrad<4>), grid, 128, st, x, cin, dy, cout, lg, chunk, dw);
-    } else {
-        dim3 grid((unsigned)(nv / chunk), 27, (cout / 16) * (cin / 16));
-        GR_LAUNCH((k_conv3d_wgrad<2>), grid, 128, st, x, cin, dy, cout, lg, chunk, dw);
-    }
+    const int lb = 3 * lg < kWgBox ? 3 * lg : kWgBox;
+    const Box bx = make_box(lg, lb);
+    const int nbox = 1 << (3 * lg - lb), pairs = (cout / 16) * (cin / 16);
+    // about four blocks per SM in all, at least one box each
+    int split = (4 * 152 + pairs - 1) / pairs;
+    if (split > nbox) split = nbox;
+    constexpr int kMost = 2 * 32 * (720 + (1 << kWgBox));
+    static const bool attr =
+        cudaFuncSetAttribute(k_conv3d_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) == cudaSuccess;
+    (void)attr;
+    const int smem = 2 * 32 * (bx.halo() + (1 << lb));
+    GR_LAUNCH_SMEM(k_conv3d_wgrad, dim3(split, pairs), 32 * kWgWarps, smem, st, x, cin, dy, cout, bx, nbox, dw);
 }
 
 void bias_grad(const __nv_bfloat16 *dy, int c, int64_t nv, float *db, cudaStream_t st)
@@ -877,12 +939,12 @@ void head(const __nv_bfloat16 *a, const float *W, const float *b, int64_t nv, fl
 void head_back(const __nv_bfloat16 *a, const float *W, const float *out, const float *tgt, int64_t nv,
                __nv_bfloat16 *da, float *dW, float *db, float *loss, cudaStream_t st)
 {
-    GR_LAUNCH(k_head_back, 152 * 4, 128, st, a, W, out, tgt, nv, da, dW, db, loss);
+    GR_LAUNCH(k_head_back, wave_grid(k_head_back, nv, kHbVox), kHbVox, st, a, W, out, tgt, nv, da, dW, db, loss);
 }
 
 void net_target(FieldPtrs fields, int64_t nv, const float *mean, const float *stdv, float *tgt, cudaStream_t st)
 {
-    GR_LAUNCH(k_net_target, cdiv(nv, 256), 256, st, fields, nv, mean, stdv, tgt);
+    GR_LAUNCH(k_net_target, cdiv(nv, 256) < 304 ? cdiv(nv, 256) : 304, 256, st, fields, nv, mean, stdv, tgt);
 }
 
 void net_output(const float *out, int64_t nv, const float *mean, const float *stdv, FieldPtrs fields,
