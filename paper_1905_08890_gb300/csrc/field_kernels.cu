@@ -104,6 +104,18 @@ __global__ void __launch_bounds__(kBlock)
     }
 }
 
+// zeros into five arrays of 2 cnt2 doubles (16-byte aligned)
+struct Ptr5 {
+    double *p[5];
+};
+__global__ void __launch_bounds__(kBlock) k_clear5(int64_t cnt2, Ptr5 f)
+{
+    pdl_begin();
+    double2 *d = reinterpret_cast<double2 *>(f.p[blockIdx.y]);
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < cnt2; t += (int64_t)gridDim.x * blockDim.x)
+        d[t] = make_double2(0.0, 0.0);
+}
+
 // ---------------------------------------------------------------- reductions
 __global__ void __launch_bounds__(kBlock) k_sum_sq(int64_t cnt, const double *__restrict__ a, const Sums sums)
 {
@@ -328,6 +340,12 @@ void deposit_add(int n, double L, int64_t np, const double *x, const double *u, 
     const int64_t blocks = (np + kBlock - 1) / kBlock;
     const int g = (int)(blocks < 0x7fffffff ? blocks : 0x7fffffff);
     GR_LAUNCH(k_deposit, g, kBlock, st, log2i(n), 1.0 / h, np, x, u, q, s0, sx, sy, sz, sig);
+}
+
+void clear5(int64_t cnt, double *const f[5], cudaStream_t st)
+{
+    const Ptr5 p{{f[0], f[1], f[2], f[3], f[4]}};
+    GR_LAUNCH(k_clear5, dim3(grid_for(cnt / 2 / 4), 5), kBlock, st, cnt / 2, p);
 }
 
 void sum_sq(int64_t cnt, const double *a, const Sums &sums, cudaStream_t st)

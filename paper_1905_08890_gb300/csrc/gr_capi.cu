@@ -1376,9 +1376,8 @@ void deposit_device(gr_ctx *c, int64_t np, const double *x, const double *u, dou
                     const gr_sources *out, bool first)
 {
     if (first) {
-        const size_t bytes = (size_t)c->n * c->n * c->n * sizeof(double);
-        double *f[5] = {out->s0, out->s[0], out->s[1], out->s[2], out->sigma};
-        for (int k = 0; k < 5; k++) cudaMemsetAsync(f[k], 0, bytes, c->st);
+        double *const f[5] = {out->s0, out->s[0], out->s[1], out->s[2], out->sigma};
+        gr::clear5((int64_t)c->n * c->n * c->n, f, c->st);
     }
     const size_t scratch = 6 * (size_t)c->n * c->n * c->n * sizeof(double);  // A_ij, which a solve makes anew
     if (gr::deposit_tiles_fit(c->n, c->L, np, mass, psi != nullptr, scratch)) {
@@ -1762,8 +1761,8 @@ gr_status gr_deposit_patches(gr_ctx *c, int npatch, const gr_patch *patch, int64
         const int N = c->n << (p + 1), n = patch[p].n;
         for (int d = 0; d < 3; d++) O[d] = (2 * (O[d] + patch[p].origin[d])) & (N - 1);
         const gr_sources &ps = patch[p].src;
-        double *f[5] = {ps.s0, ps.s[0], ps.s[1], ps.s[2], ps.sigma};
-        for (int k = 0; k < 5; k++) cudaMemsetAsync(f[k], 0, (size_t)n * n * n * sizeof(double), c->st);
+        double *const f[5] = {ps.s0, ps.s[0], ps.s[1], ps.s[2], ps.sigma};
+        gr::clear5((int64_t)n * n * n, f, c->st);
         const gr::PSetSrc out{{f[0], f[1], f[2], f[3], f[4]}};
         if (listed) gr::patch_deposit_list(np, c->plist, c->pcount, x, u, mass, c->L, N, O, n, out, c->st);
         else gr::patch_deposit(np, x, u, mass, c->L, N, O, n, out, c->st);

@@ -431,6 +431,9 @@ void dfs_weight(int n, const double *psi, const double *apsi, float *wh, float *
 void dfs_store(int n, const float *uh, const float *ul, const double *sum, int dev, double *out, cudaStream_t st);
 
 // ---- sources, coefficients, layouts (field_kernels.cu) ---------------------
+// zeros into the five source arrays of cnt (even) doubles each: one launch (five memsets cost a small
+// deposit of 12345 particles on 32^3 cells 28.7 us, so 13.0)
+void clear5(int64_t cnt, double *const f[5], cudaStream_t st);
 // the deposit kernel, one thread per particle, adding to the five arrays (no zeroing)
 void deposit_add(int n, double L, int64_t np, const double *x, const double *u, double mass, double *s0, double *sx,
                  double *sy, double *sz, double *sig, cudaStream_t st);
