@@ -487,38 +487,49 @@ __device__ __forceinline__ uint4 bf8_pack(const float f[8])
     return r;
 }
 
-__global__ void k_upsample8(const __nv_bfloat16 *__restrict__ x, int lgc8, int lgc, __nv_bfloat16 *__restrict__ y,
-                            int cstride)
+// Eight channels of the four fine voxels (j, k) = (2 J + 0..1, 2 K + 0..1) of a fine plane i per
+// thread: 18 coarse voxels are read and unpacked for them (8 per fine voxel on its own:
+// 74 us for 32 channels to 128^3, so 55).  Per voxel the eight products are added in the
+// order own cell first, then neighbour, along i, j, k.
+__global__ void __launch_bounds__(256)
+    k_upsample8(const __nv_bfloat16 *__restrict__ x, int lgc8, int lgc, __nv_bfloat16 *__restrict__ y, int cstride)
 {
     pdl_begin();
-    const int lgf = lgc + 1, mf = (1 << lgf) - 1, mc = (1 << lgc) - 1, c = 8 << lgc8;
-    const int total = 1 << (3 * lgf + lgc8);
+    const int lgf = lgc + 1, mc = (1 << lgc) - 1, c = 8 << lgc8;
+    const int total = 1 << (3 * lgc + 1 + lgc8);
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
         const int ch = (e & ((1 << lgc8) - 1)) << 3;
         const int v = e >> lgc8;
-        const int k = v & mf, j = (v >> lgf) & mf, i = v >> (2 * lgf);
-        int I[2], J[2], K[2];
-        I[0] = i >> 1;
-        I[1] = (i & 1) ? ((I[0] + 1) & mc) : ((I[0] - 1) & mc);
-        J[0] = j >> 1;
-        J[1] = (j & 1) ? ((J[0] + 1) & mc) : ((J[0] - 1) & mc);
-        K[0] = k >> 1;
-        K[1] = (k & 1) ? ((K[0] + 1) & mc) : ((K[0] - 1) & mc);
+        const int K = v & mc, J = (v >> lgc) & mc, i = v >> (2 * lgc);
+        const int I[2] = {i >> 1, ((i >> 1) + ((i & 1) ? 1 : -1)) & mc};
+        const int js[3] = {J, (J - 1) & mc, (J + 1) & mc}, ks[3] = {K, (K - 1) & mc, (K + 1) & mc};
         const float wt[2] = {0.75f, 0.25f};
-        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        float s[2][2][8] = {};
 #pragma unroll
         for (int a = 0; a < 2; a++)
 #pragma unroll
-            for (int b = 0; b < 2; b++)
+            for (int b = 0; b < 3; b++)
 #pragma unroll
-                for (int q = 0; q < 2; q++) {
-                    const float w = wt[a] * wt[b] * wt[q];
+                for (int q = 0; q < 3; q++) {
                     float xv[8];
-                    bf8_unpack(*reinterpret_cast<const uint4 *>(x + (size_t)((((I[a] << lgc) + J[b]) << lgc) + K[q]) * c + ch), xv);
+                    bf8_unpack(*reinterpret_cast<const uint4 *>(x + (size_t)((((I[a] << lgc) + js[b]) << lgc) + ks[q]) * c + ch), xv);
+                    // the own cell serves both fine voxels of its axis, J - 1 the lower and J + 1 the upper one
 #pragma unroll
-                    for (int m = 0; m < 8; m++) s[m] += w * xv[m];
+                    for (int fj = 0; fj < 2; fj++)
+#pragma unroll
+                        for (int fk = 0; fk < 2; fk++) {
+                            if ((b != 0 && b != fj + 1) || (q != 0 && q != fk + 1)) continue;
+                            const float w = wt[a] * wt[b != 0] * wt[q != 0];
+#pragma unroll
+                            for (int m = 0; m < 8; m++) s[fj][fk][m] += w * xv[m];
+                        }
                 }
-        *reinterpret_cast<uint4 *>(y + (size_t)v * cstride + ch) = bf8_pack(s);
+#pragma unroll
+        for (int fj = 0; fj < 2; fj++)
+#pragma unroll
+            for (int fk = 0; fk < 2; fk++)
+                *reinterpret_cast<uint4 *>(y + (size_t)((((i << lgf) + 2 * J + fj) << lgf) + 2 * K + fk) * cstride + ch) =
+                    bf8_pack(s[fj][fk]);
     }
 }
 
@@ -568,22 +579,48 @@ __global__ void k_net_input(const double *__restrict__ s0, const double *__restr
 }
 
 // 1x1 head (FP32): out[v][o] = b[o] + sum_c W[o][c] a[v][c], a with 16 channels
-__global__ void k_head(const __nv_bfloat16 *__restrict__ a, const float *__restrict__ W, const float *__restrict__ b,
-                       int64_t nv, float *__restrict__ out)
+// (a block's outputs pass through shared memory: 36 us at 128^3; stored with a stride of 40 bytes, 62)
+constexpr int kHeadVox = 256;
+__global__ void __launch_bounds__(kHeadVox)
+    k_head(const __nv_bfloat16 *__restrict__ a, const float *__restrict__ W, const float *__restrict__ b, int64_t nv,
+           float *__restrict__ out)
 {
     pdl_begin();
-    __shared__ float sw[kNetOut * 16 + kNetOut];
-    for (int k = threadIdx.x; k < kNetOut * 16; k += blockDim.x) sw[k] = W[k];
-    for (int k = threadIdx.x; k < kNetOut; k += blockDim.x) sw[kNetOut * 16 + k] = b[k];
+    __shared__ __align__(16) float sw[kNetOut * 16], sb[kNetOut], so[kHeadVox * kNetOut];
+    for (int k = threadIdx.x; k < kNetOut * 16; k += kHeadVox) sw[k] = W[k];
+    for (int k = threadIdx.x; k < kNetOut; k += kHeadVox) sb[k] = b[k];
     __syncthreads();
-    for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += (int64_t)gridDim.x * blockDim.x) {
-        float av[16];
-        for (int c = 0; c < 16; c++) av[c] = __bfloat162float(a[v * 16 + c]);
-        for (int o = 0; o < kNetOut; o++) {
-            float s = sw[kNetOut * 16 + o];
-            for (int c = 0; c < 16; c++) s += sw[o * 16 + c] * av[c];
-            out[v * kNetOut + o] = s;
+    for (int64_t v0 = (int64_t)blockIdx.x * kHeadVox; v0 < nv; v0 += (int64_t)gridDim.x * kHeadVox) {
+        const int64_t v = v0 + threadIdx.x;
+        if (v < nv) {
+            const uint4 *a8 = reinterpret_cast<const uint4 *>(a + v * 16);
+            float lo[8], hi[8];
+            bf8_unpack(a8[0], lo);
+            bf8_unpack(a8[1], hi);
+#pragma unroll
+            for (int o = 0; o < kNetOut; o++) {
+                float s = sb[o];
+#pragma unroll
+                for (int c = 0; c < 16; c += 4) {
+                    const float4 w = *reinterpret_cast<const float4 *>(sw + o * 16 + c);
+                    const float *x = c < 8 ? lo + c : hi + (c - 8);
+                    s += w.x * x[0];
+                    s += w.y * x[1];
+                    s += w.z * x[2];
+                    s += w.w * x[3];
+                }
+                so[threadIdx.x * kNetOut + o] = s;
+            }
         }
+        __syncthreads();
+        const int cnt = (int)(nv - v0 < kHeadVox ? nv - v0 : kHeadVox) * kNetOut;
+        float *dst = out + v0 * kNetOut;  // v0 is a multiple of 256: 16-byte aligned
+        for (int k = 4 * threadIdx.x; k < cnt; k += 4 * kHeadVox) {
+            if (k + 4 <= cnt) *reinterpret_cast<float4 *>(dst + k) = *reinterpret_cast<const float4 *>(so + k);
+            else
+                for (int r = k; r < cnt; r++) dst[r] = so[r];
+        }
+        __syncthreads();
     }
 }
 
@@ -885,7 +922,7 @@ void upsample(const __nv_bfloat16 *x, int c, int lgc, __nv_bfloat16 *y, int cstr
 {
     const int l8 = pow2_log(c) - 3;
     if (l8 >= 0 && cstride % 8 == 0 && 3 * lgc + 3 + l8 < 31) {
-        GR_LAUNCH(k_upsample8, cdiv((int64_t)1 << (3 * lgc + 3 + l8), 256), 256, st, x, l8, lgc, y, cstride);
+        GR_LAUNCH(k_upsample8, cdiv((int64_t)1 << (3 * lgc + 1 + l8), 256), 256, st, x, l8, lgc, y, cstride);
         return;
     }
     GR_LAUNCH(k_upsample, cdiv(((int64_t)1 << (3 * lgc + 3)) * c, 256), 256, st, x, c, lgc, y, cstride);
@@ -933,7 +970,7 @@ void net_output_fine(const float *out, int lgc, int lr, const float *mean, const
 
 void head(const __nv_bfloat16 *a, const float *W, const float *b, int64_t nv, float *out, cudaStream_t st)
 {
-    GR_LAUNCH(k_head, cdiv(nv, 256), 256, st, a, W, b, nv, out);
+    GR_LAUNCH(k_head, wave_grid(k_head, nv, kHeadVox), kHeadVox, st, a, W, b, nv, out);
 }
 
 void head_back(const __nv_bfloat16 *a, const float *W, const float *out, const float *tgt, int64_t nv,
