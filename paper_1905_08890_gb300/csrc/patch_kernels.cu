@@ -197,6 +197,47 @@ __device__ __forceinline__ df p_cell_df(const PPatch &P, df lam2, int i, int j, 
     return df_cell<KIND>(nh, nl, {P.uh[c], P.ul[c]}, f, a, b, P.cpr, P.c5, &mj, inv);
 }
 
+// h^2 lambda as a double-float, formed once per block
+__device__ __forceinline__ df p_lambda(const PPatch &P)
+{
+    __shared__ df s_lam;
+    if (!P.lam) return {0.0f, 0.0f};
+    if (threadIdx.x == 0) s_lam = split_double(*P.lam * P.h2);
+    __syncthreads();
+    return s_lam;
+}
+
+// p_cell_df of the cells (i, j, k) and (i, j, k + 1), k even, with vector loads
+template <int KIND>
+__device__ __forceinline__ void p_pair_df(const PPatch &P, df lam2, int i, int j, int k, df (&e)[2])
+{
+    const int m = P.m, mm = m * m;
+    const int c = gxi(m, i, j, k);  // even
+    const int nb[4] = {c + mm, c - mm, c + m, c - m};
+    auto two = [](const float *q) { return *reinterpret_cast<const float2 *>(q); };
+    float nh[2][6], nl[2][6];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const float2 h = two(P.uh + nb[q]), l = two(P.ul + nb[q]);
+        nh[0][q] = h.x, nh[1][q] = h.y;
+        nl[0][q] = l.x, nl[1][q] = l.y;
+    }
+    const float2 uh = two(P.uh + c), ul = two(P.ul + c), fh = two(P.fh + c), fl = two(P.fl + c);
+    nh[0][4] = uh.y, nl[0][4] = ul.y;
+    nh[0][5] = P.uh[c - 1], nl[0][5] = P.ul[c - 1];
+    nh[1][4] = P.uh[c + 2], nl[1][4] = P.ul[c + 2];
+    nh[1][5] = uh.x, nl[1][5] = ul.x;
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+        df f = q ? df{fh.y, fl.y} : df{fh.x, fl.x};
+        if (P.lam && !p_covered(P, i, j, k + q)) f = df_add(f, lam2);
+        const df a = KIND == KPOISSON ? df{0.0f, 0.0f} : df{P.ah[c + q], P.al[c + q]};
+        const df b = KIND == KPSI ? df{P.bh[c + q], P.bl[c + q]} : df{0.0f, 0.0f};
+        float mj = 0.0f, inv;
+        e[q] = df_cell<KIND>(nh[q], nl[q], q ? df{uh.y, ul.y} : df{uh.x, ul.x}, f, a, b, P.cpr, P.c5, &mj, &inv);
+    }
+}
+
 // right-hand side of a patch cell: f, plus the solvability constant lambda
 // where the child patch does not cover the cell
 __device__ __forceinline__ double p_rhs(const PPatch &P, int i, int j, int k)
@@ -512,21 +553,27 @@ __global__ void __launch_bounds__(kBlock) k_presid(PPatch P, double *__restrict_
 {
     pdl_begin();
     const int64_t N = (int64_t)1 << (3 * P.lgn);
-    df lam2 = {0.0f, 0.0f};
-    if (DF && P.lam) lam2 = split_double(*P.lam * P.h2);
     double s2 = 0.0;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N; t += (int64_t)gridDim.x * blockDim.x) {
-        int i, j, k;
-        p_cell(P.lgn, t, i, j, k);
-        double e;
-        if (DF) {
-            float inv;
-            e = join_double(p_cell_df<KIND>(P, lam2, i, j, k, &inv)) * P.ih2;
-        } else {
-            e = p_op<KIND>(P, i, j, k) - p_rhs(P, i, j, k);
+    if (DF) {  // two cells (k, k + 1) per thread: 25 us at 128^3 against 29.5 for one, bound by issue and the FP64 pipe
+        const df lam2 = p_lambda(P);
+        for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N / 2; t += (int64_t)gridDim.x * blockDim.x) {
+            int i, j, k;
+            p_cell(P.lgn, 2 * t, i, j, k);
+            df d[2];
+            p_pair_df<KIND>(P, lam2, i, j, k, d);
+            const double e0 = join_double(d[0]) * P.ih2, e1 = join_double(d[1]) * P.ih2;
+            *reinterpret_cast<double2 *>(eps + gxi(P.m, i, j, k)) = make_double2(e0, e1);
+            s2 += e0 * e0;
+            s2 += e1 * e1;
         }
-        eps[gxi(P.m, i, j, k)] = e;
-        s2 += e * e;
+    } else {
+        for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N; t += (int64_t)gridDim.x * blockDim.x) {
+            int i, j, k;
+            p_cell(P.lgn, t, i, j, k);
+            const double e = p_op<KIND>(P, i, j, k) - p_rhs(P, i, j, k);
+            eps[gxi(P.m, i, j, k)] = e;
+            s2 += e * e;
+        }
     }
     block_sum2(s2, 0.0, sums);
 }
@@ -667,12 +714,11 @@ __device__ __forceinline__ void shell_cell(int q, int nc, int n, int in[3], int 
 
 template <int PARENT, bool DF>
 __global__ void __launch_bounds__(kBlock) k_reflux(PBase B, PPatch par, PPatch ch, int o0, int o1, int o2, int n,
-                                                   double hc, double *__restrict__ flux)
+                                                   double ihc, double *__restrict__ flux)
 {
     pdl_begin();
     const int nc = n / 2, m = n + 2 * PG;
     const int nq = 6 * nc * nc;
-    const double hf = 0.5 * hc;
     for (int q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x) {
         int in[3], out[3], fi[4][3], fg[4][3];
         shell_cell(q, nc, n, in, out, fi, fg);
@@ -686,13 +732,13 @@ __global__ void __launch_bounds__(kBlock) k_reflux(PBase B, PPatch par, PPatch c
             uin = b_u<PARENT>(B, ii, ij, ik);
             uout = b_u<PARENT>(B, oi, oj, ok);
         }
-        const double Tc = (uin - uout) / hc;
+        const double Tc = (uin - uout) * ihc;
         double Tf = 0.0;
         for (int e = 0; e < 4; e++)
-            Tf += (pu_get<DF>(ch, gxi(m, fi[e][0], fi[e][1], fi[e][2])) -
-                   pu_get<DF>(ch, gxi(m, fg[e][0], fg[e][1], fg[e][2]))) / hf;
-        Tf *= 0.25;
-        const double corr = -(Tf - Tc) / hc;
+            Tf += pu_get<DF>(ch, gxi(m, fi[e][0], fi[e][1], fi[e][2])) -
+                  pu_get<DF>(ch, gxi(m, fg[e][0], fg[e][1], fg[e][2]));
+        Tf *= 0.5 * ihc;  // mean of four over hc / 2
+        const double corr = (Tc - Tf) * ihc;
         const double d = corr - flux[q];
         flux[q] = corr;
         if (PARENT == 0) {
@@ -873,12 +919,28 @@ __device__ __forceinline__ double aa_of(const double A[6])
     return A[0] * A[0] + A[1] * A[1] + A[2] * A[2] + 2.0 * (A[3] * A[3] + A[4] * A[4] + A[5] * A[5]);
 }
 
+// alpha psi psi^-7 on the cells whose neighbours k_pset differences for B^i (the interior
+// and one ghost layer): once per cell, where each of its six neighbours forming it
+// took 317 us per equation at 128^3; now 41 and 50
+__global__ void __launch_bounds__(kBlock)
+    k_pratio(int n, const double *__restrict__ psi, const double *__restrict__ apsi, double *__restrict__ r)
+{
+    pdl_begin();
+    const int m = n + 2 * PG, w = n + 2, N = w * w * w;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < N; t += gridDim.x * blockDim.x) {
+        const int k = t % w, j = t / w % w, i = t / (w * w);
+        const int q = gxi(m, i - 1, j - 1, k - 1);
+        const double p = psi[q], p2 = p * p, p4 = p2 * p2;
+        r[q] = apsi[q] * recip64(p4 * p2 * p);
+    }
+}
+
 // Right-hand side and coefficients of equation eq (solve order) on a patch's
 // interior (ghosted f, c0, c1), with block sums of the square of the
 // reference quantity: the momentum sources 8 pi (s_i - smean); the
 // divergence sources -div/4; psi: c0 = s0, c1 = AA, f = 0 (reference s0);
 // alpha psi: c0 = m, c1 = 1/(6 + h^2 m), f = m - psi^5 Kdot (reference psi^5 Kdot); B^i:
-// 2 d_j (alpha psi psi^-7 A^ij).  G: ghosted fields in the order V_x V_y V_z
+// 2 d_j (alpha psi psi^-7 A^ij), c0 holding alpha psi psi^-7.  G: ghosted fields in the order V_x V_y V_z
 // U psi apsi B^x B^y B^z b.
 __global__ void __launch_bounds__(kBlock)
     k_pset(int eq, int lgn, double nh, PSetSrc S, PSetFld G, const double *__restrict__ A6, double smean, double K2,
@@ -889,7 +951,7 @@ __global__ void __launch_bounds__(kBlock)
     const int64_t N = (int64_t)1 << (3 * lgn);
     const int m = (1 << lgn) + 2 * PG;
     const int64_t M = (int64_t)m * m * m;
-    const double i2h = 0.5 * nh;
+    const double i2h = 0.5 * nh, h2 = 1.0 / (nh * nh);
     double s2 = 0.0;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N; t += (int64_t)gridDim.x * blockDim.x) {
         int i, j, k;
@@ -915,12 +977,14 @@ __global__ void __launch_bounds__(kBlock)
             double A[6];
             for (int q = 0; q < 6; q++) A[q] = A6[q * M + g];
             const double aa = aa_of(A);
-            const double p = G.g[4][g], p2 = p * p, p4 = p2 * p2, p8 = p4 * p4;
-            c0[g] = 2.0 * kPi / p2 * (S.s[0][t] + 2.0 * S.s[4][t] / p4) + 0.875 * aa / p8 + (5.0 / 12.0) * p4 * K2;
-            c1[g] = 1.0 / (6.0 + c0[g] / (nh * nh));  // the inverse diagonal of the relaxation
+            const double p = G.g[4][g], p2 = p * p, p4 = p2 * p2;
+            const double i2 = recip64(p2), i4 = i2 * i2;
+            const double mm = 2.0 * kPi * i2 * (S.s[0][t] + 2.0 * S.s[4][t] * i4) + 0.875 * aa * (i4 * i4) + (5.0 / 12.0) * p4 * K2;
+            c0[g] = mm;
+            c1[g] = recip64(6.0 + mm * h2);  // the inverse diagonal of the relaxation
             const double fk = -p4 * p * Kdot;
             s2 += fk * fk;
-            f[g] = fk + c0[g];
+            f[g] = fk + mm;
         } else {
             const int tab[3][3] = {{0, 3, 4}, {3, 1, 5}, {4, 5, 2}};
             double s = 0.0;
@@ -929,8 +993,7 @@ __global__ void __launch_bounds__(kBlock)
                     int c[3] = {i, j, k};
                     c[l] += sg;
                     const int64_t q = gxi(m, c[0], c[1], c[2]);
-                    const double p = G.g[4][q], p2 = p * p, p4 = p2 * p2;
-                    s += (double)sg * G.g[5][q] / (p4 * p2 * p) * A6[tab[eq - 6][l] * M + q];
+                    s += (double)sg * c0[q] * A6[tab[eq - 6][l] * M + q];  // c0 = alpha psi psi^-7 (k_pratio)
                 }
             f[g] = 2.0 * s * i2h;
             s2 += f[g] * f[g];
@@ -1030,7 +1093,7 @@ void patch_gs(int kind, const PPatch &P, bool pdf, int color, cudaStream_t st)
 void patch_resid(int kind, const PPatch &P, bool pdf, double *eps, const Sums &sums, cudaStream_t st)
 {
     const int64_t work = (int64_t)1 << (3 * P.lgn);
-#define GR_PRES(K, D) GR_LAUNCH((k_presid<K, D>), wave_grid(k_presid<K, D>, work), kBlock, st, P, eps, sums)
+#define GR_PRES(K, D) GR_LAUNCH((k_presid<K, D>), wave_grid(k_presid<K, D>, D ? work / 2 : work), kBlock, st, P, eps, sums)
     if (pdf) {
         if (kind == KPOISSON) GR_PRES(KPOISSON, true);
         else if (kind == KHELM) GR_PRES(KHELM, true);
@@ -1110,8 +1173,11 @@ void patch_reflux(int parent_fmt, const PBase &B, const PPatch &par, const PPatc
                   double hc, double *flux, cudaStream_t st)
 {
     const int n = 1 << ch.lgn, nc = n / 2;
-    const int g = blocks_for((int64_t)6 * nc * nc);
-#define GR_RFX(F, D) GR_LAUNCH((k_reflux<F, D>), g, kBlock, st, B, par, ch, o[0], o[1], o[2], n, hc, flux)
+    // 64 threads a block, so that the 24576 faces of a 128^3 patch reach every SM's FP64 pipe; 1 / hc
+    // formed here: 10 us (with 96 blocks and six divisions a face 13.7)
+    const int g = (6 * nc * nc + 63) / 64;
+    const double ihc = 1.0 / hc;
+#define GR_RFX(F, D) GR_LAUNCH((k_reflux<F, D>), g, 64, st, B, par, ch, o[0], o[1], o[2], n, ihc, flux)
     if (pdf) {
         if (parent_fmt < 0) GR_RFX(0, true);
         else if (parent_fmt == PB_SPLIT) GR_RFX(PB_SPLIT, true);
@@ -1170,6 +1236,8 @@ void patch_aij(int n, double nh, const PSetFld &G, double *A6, cudaStream_t st)
 void patch_setup(int eq, int n, double nh, const PSetSrc &S, const PSetFld &G, const double *A6, double smean,
                 double K2, double Kdot, double *f, double *c0, double *c1, const Sums &sums, cudaStream_t st)
 {
+    if (eq >= 6 && eq <= 8)
+        GR_LAUNCH(k_pratio, wave_grid(k_pratio, (int64_t)(n + 2) * (n + 2) * (n + 2)), kBlock, st, n, G.g[4], G.g[5], c0);
     const int g = wave_grid(k_pset, (int64_t)n * n * n);
     GR_LAUNCH(k_pset, g, kBlock, st, eq, lg2(n), nh, S, G, A6, smean, K2, Kdot, f, c0, c1, sums);
 }
