@@ -49,11 +49,13 @@ __device__ __forceinline__ void stv(float *p, const float (&v)[W])
     else *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
 }
 
-// blocks per SM the residual kernel is compiled for (registers per thread)
-template <int KIND, int W>
+// blocks per SM the residual kernel is compiled for (registers per thread).
+// BIG (Poisson from 512^3, whose arrays come from HBM): fewer blocks with more loads in flight each,
+// 504 against 548 us at 512^3; at 256^3, mostly in L2, three blocks are faster (70 against 72 us)
+template <int KIND, int W, bool BIG>
 constexpr int resid_min_blocks()
 {
-    return W == 4 ? (KIND == KPSI ? 2 : 3) : (KIND == KPOISSON ? 5 : (KIND == KHELM ? 4 : 3));
+    return W == 4 ? (KIND == KPSI || BIG ? 2 : 3) : (KIND == KPOISSON ? 5 : (KIND == KHELM ? 4 : 3));
 }
 
 // eps = L(u) - f on the finest level; writes r32 = -eps and, for the psi
@@ -69,8 +71,8 @@ constexpr int resid_min_blocks()
 // which starts from e = 0: e_red = -h^2 r / 6 (Poisson) or -h^2 r / (6 + h^2 m).
 // SHIFT (Poisson with nested patches): every cell's right-hand side is
 // f + fshift[0] (the solvability constant), i.e. h^2 f + fshift[0] * fsh_scale.
-template <int KIND, int W, bool SHIFT = false>
-__global__ void __launch_bounds__(kBlock, (resid_min_blocks<KIND, W>()))
+template <int KIND, int W, bool SHIFT = false, bool BIG = false>
+__global__ void __launch_bounds__(kBlock, (resid_min_blocks<KIND, W, BIG>()))
     k_df_resid(int lgn, const float *__restrict__ uh, const float *__restrict__ ul, const float *__restrict__ fh,
                const float *__restrict__ fl, const float *__restrict__ ah, const float *__restrict__ al,
                const float *__restrict__ bh, const float *__restrict__ bl, df cpr, float c5, float ih2,
@@ -157,14 +159,10 @@ __global__ void __launch_bounds__(kBlock, (resid_min_blocks<KIND, W>()))
             }
             if (c == 0 && e32) {
                 float g[W];
-                if (KIND == KHELM) {
-                    ldv<W>(inv_in + own, g);
-                } else {
+                if (KIND == KHELM) ldv<W>(inv_in + own, g);
 #pragma unroll
-                    for (int e = 0; e < W; e++) g[e] = KIND == KPOISSON ? 1.0f / 6.0f : iv[e];
-                }
-#pragma unroll
-                for (int e = 0; e < W; e++) g[e] *= sh[e];
+                for (int e = 0; e < W; e++)
+                    g[e] = KIND == KPOISSON ? first_red(rr[e], (float)fsh_scale) : sh[e] * (KIND == KHELM ? g[e] : iv[e]);
                 stv<W>(e32 + own, g);
             }
         }
@@ -254,17 +252,19 @@ void df_resid(int kind, int n, const float *uh, const float *ul, const float *fh
     const df cpr = df_from_double_host(2.0 * kPi * rho * h2);
     const float c5 = (float)(10.0 * kPi * rho * h2), ih2 = (float)(1.0 / h2), ih2_ref = (float)(1.0 / (h2 * ref));
     int g = 0;
-#define GR_DF_RESID(K, W, S)                                                                                     \
+#define GR_DF_RESID(K, W, ...)                                                                                   \
     do {                                                                                                         \
-        g = wave_grid(k_df_resid<K, W, S>, threads);                                                             \
-        GR_LAUNCH((k_df_resid<K, W, S>), g, kBlock, st, lgn, uh, ul, fh, fl, ah, al, bh, bl, cpr, c5, ih2,       \
+        g = wave_grid(k_df_resid<K, W, __VA_ARGS__>, threads);                                                   \
+        GR_LAUNCH((k_df_resid<K, W, __VA_ARGS__>), g, kBlock, st, lgn, uh, ul, fh, fl, ah, al, bh, bl, cpr, c5, ih2, \
                   ih2_ref, r32, m32, inv32, inv_in, e32, sums, rev, fshift, h2);                             \
     } while (0)
     if (kind == KPOISSON && fshift) {
-        if (w == 4) GR_DF_RESID(KPOISSON, 4, true);
+        if (n >= 512) GR_DF_RESID(KPOISSON, 4, true, true);
+        else if (w == 4) GR_DF_RESID(KPOISSON, 4, true);
         else GR_DF_RESID(KPOISSON, 2, true);
     } else if (kind == KPOISSON) {
-        if (w == 4) GR_DF_RESID(KPOISSON, 4, false);
+        if (n >= 512) GR_DF_RESID(KPOISSON, 4, false, true);
+        else if (w == 4) GR_DF_RESID(KPOISSON, 4, false);
         else GR_DF_RESID(KPOISSON, 2, false);
     } else if (kind == KHELM) {
         if (w == 4) GR_DF_RESID(KHELM, 4, false);

@@ -575,8 +575,15 @@ int next_dir(gr_ctx *c)
 // How a correction V-cycle finds its top level's e: zero (cleared here), the
 // first red relaxation from zero already made (by the fine residual kernel;
 // the black cells are then not read before they are written), or a given
-// initial e (full multigrid).
-enum Start { START_ZERO = 0, START_RED_DONE = 1, START_GIVEN = 2 };
+// initial e (full multigrid).  START_FROM_R: as START_RED_DONE, but the red
+// values are formed from r by the black pass that follows (red_from_r).
+enum Start { START_ZERO = 0, START_RED_DONE = 1, START_GIVEN = 2, START_FROM_R = 3 };
+
+// Whether a correction cycle may start from r alone: a second red pass has to
+// overwrite the red values before anything else reads them.  It spares the residual
+// kernel 2 of the 22 bytes per cell it moves (504 -> 479 us at 512^3; the black pass, whose
+// neighbours are then not in L2, goes from 117 to 128).  Smaller finest levels pre-smooth in one launch.
+bool red_from_r(const Level &F, int kind32, int nu1) { return kind32 == KPOISSON && nu1 >= 2 && !F.e2 && F.n >= 128; }
 
 // One FP32 correction V-cycle on lev[*].e with right-hand side lev[top].r,
 // top = the finest level unless given (full multigrid's coarser cycles, all
@@ -674,6 +681,11 @@ void vcycle32(gr_ctx *c, int kind32, int nu1, int nu2, Start start, float *uh = 
                 gr::sweep_colour<float>(kind32, F.n, F.e, F.r, F.m, F.inv, F.h2, F.ih2, 0.0, 0, c->st, dir_of(F));
             });
         timed(c, cls(GR_PROF_RESTRICT), [&] { level_down(top, start == START_ZERO); });
+    } else if (start == START_FROM_R) {
+        timed(c, cls(GR_PROF_SWEEP32), [&] {
+            gr::sweep_black_from_r(F.n, F.e, F.r, F.h2, c->st, dir_of(F));
+            smooth(F, nu1 - 1);
+        });
     } else if (start == START_RED_DONE && nu1 > 0) {
         if (!fused3(nu1, 1)) {
             timed(c, cls(GR_PROF_SWEEP32), [&] {
@@ -1163,7 +1175,7 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
     const int64_t N = (int64_t)F.n * F.n * F.n;
     // the double-float residual also makes the first red pass of the next
     // cycle, and the last black pass adds the correction to u
-    const bool red = dfm && o->nu1 > 0;
+    const bool red = dfm && o->nu1 > 0, from_r = red && red_from_r(c->lev[c->nlev - 1], in.kind32, o->nu1);
     const bool fuse_update = dfm && o->nu2 > 0 && F.n >= 8;
     // full multigrid start: the first correction of the equation (mixed modes, coarse tail present)
     const bool fmg = o->fmg != 0 && (o->prec == GR_PREC_MIXED || dfm) && c->nlev - 1 > 3 && c->tail_on;
@@ -1212,7 +1224,7 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
     double rlev[GR_MAX_PATCHES + 1] = {};
     // the base residual and, with patches, the largest of all levels' (rlev: each level's)
     auto queue_norm = [&] {
-        if (dfm) df_norm(c, in, rho, red, (patches && in.poisson) ? c->pdev : nullptr);
+        if (dfm) df_norm(c, in, rho, red && !from_r, (patches && in.poisson) ? c->pdev : nullptr);
         else if (mixed) mixed_norm(c, in, rho);
         else norm64(c, in.kind, rho, nullptr);
     };
@@ -1259,7 +1271,7 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
         if (mixed) {
             if (in.kind == KPSI) restrict_coefs32(c);
             const bool full = fmg && cyc == 0;
-            const Start start = red ? START_RED_DONE : START_ZERO;
+            const Start start = from_r ? START_FROM_R : (red ? START_RED_DONE : START_ZERO);
             if (fuse_update) {
                 if (full) fmg32(c, in.kind32, o->nu1, o->nu2, c->dfu, c->dfu + N);
                 else vcycle32(c, in.kind32, o->nu1, o->nu2, start, c->dfu, c->dfu + N);

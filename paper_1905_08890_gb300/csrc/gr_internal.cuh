@@ -150,6 +150,9 @@ struct Sums {
 };
 
 #ifdef __CUDACC__
+// the first red relaxation of a Poisson correction from e = 0 (rounded as if stored: not contracted into the sum it enters)
+__device__ __forceinline__ float first_red(float r, float h2) { return __fmul_rn(__fmul_rn(-h2, r), 1.0f / 6.0f); }
+
 // 1/x by Newton's iteration r <- r + r (1 - x r) from the hardware's 20-bit
 // estimate: two steps leave about one unit in the last place
 __device__ __forceinline__ double recip64(double x)
@@ -276,6 +279,9 @@ __device__ __forceinline__ void block_sum2f(float a, float b, const Sums &S)
 template <typename T>
 void sweep_colour(int kind, int n, T *u, const T *f, const T *c0, const T *c1, double h2, double ih2, double rho,
                   int color, cudaStream_t st, int rev = 0);
+// KPOISSON, n >= 8: the black pass that follows the first red one from e = 0, with the red values
+// -h^2 r / 6 formed here from r instead of read from e (whose red half nothing need write)
+void sweep_black_from_r(int n, float *e, const float *r, double h2, cudaStream_t st, int rev = 0);
 
 // Residual eps = L(u) - f of the fine level restricted to the coarse level.
 // Correction form (fas = 0): fc = -R eps, uc = 0.  FAS (fas = 1, KPSI):

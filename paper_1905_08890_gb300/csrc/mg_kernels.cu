@@ -139,7 +139,9 @@ __global__ void __launch_bounds__(kBlock)
 // rows (i +- 1, j), (i, j +- 1) and the own row of the other colour are read
 // as float4; the shifted own-row neighbour q + (p ? 1 : -1) takes one extra
 // scalar load.  Needs n >= 8 (rows of at least four half-indices).
-template <int KIND>
+// FROM_R (KPOISSON, black, the first pass after the first red one from e = 0): the red
+// values are formed from the right-hand side, -h^2 r / 6, so that nobody writes them.
+template <int KIND, bool FROM_R = false>
 __global__ void __launch_bounds__(kBlock) k_sweep4(int lgn, float *__restrict__ u, const float *__restrict__ f,
                                                    const float *__restrict__ c1, float h2, int color, int rev)
 {
@@ -148,8 +150,13 @@ __global__ void __launch_bounds__(kBlock) k_sweep4(int lgn, float *__restrict__ 
     const int64_t half = (int64_t)1 << (3 * lgn - 1);
     const int64_t off = color ? half : 0;
     float *__restrict__ own = u + off;
-    const float *__restrict__ oth = u + (half - off);
+    const float *__restrict__ oth = (FROM_R ? f : u) + (half - off);
     const int64_t nvec = half >> 2;
+    auto other = [&](int64_t id) {
+        float4 a = *reinterpret_cast<const float4 *>(oth + id);
+        if (FROM_R) a = make_float4(first_red(a.x, h2), first_red(a.y, h2), first_red(a.z, h2), first_red(a.w, h2));
+        return a;
+    };
     for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nvec; v += (int64_t)gridDim.x * blockDim.x) {
         const int64_t t = (rev ? nvec - 1 - v : v) << 2;
         const int q = (int)(t & mh);
@@ -163,13 +170,14 @@ __global__ void __launch_bounds__(kBlock) k_sweep4(int lgn, float *__restrict__ 
         const int64_t rj = (int64_t)i << (lgn + lgh);
         const int64_t rjp = rj + ((int64_t)((j + 1) & mn) << lgh);
         const int64_t rjm = rj + ((int64_t)((j - 1) & mn) << lgh);
-        const float4 A = *reinterpret_cast<const float4 *>(oth + rip + q);
-        const float4 B = *reinterpret_cast<const float4 *>(oth + rim + q);
-        const float4 C = *reinterpret_cast<const float4 *>(oth + rjp + q);
-        const float4 D = *reinterpret_cast<const float4 *>(oth + rjm + q);
-        const float4 E = *reinterpret_cast<const float4 *>(oth + r0 + q);
+        const float4 A = other(rip + q);
+        const float4 B = other(rim + q);
+        const float4 C = other(rjp + q);
+        const float4 D = other(rjm + q);
+        const float4 E = other(r0 + q);
         const float4 F = *reinterpret_cast<const float4 *>(f + off + t);
-        const float x = oth[r0 + ((q + (p ? 4 : -1)) & mh)];
+        float x = oth[r0 + ((q + (p ? 4 : -1)) & mh)];
+        if (FROM_R) x = first_red(x, h2);
         const float4 Sh = p ? make_float4(E.y, E.z, E.w, x) : make_float4(x, E.x, E.y, E.z);
         float4 nb;
         nb.x = A.x + B.x + C.x + D.x + E.x + Sh.x;
@@ -843,6 +851,13 @@ void sweep_colour(int kind, int n, T *u, const T *f, const T *c0, const T *c1, d
         GR_LAUNCH((k_sweep<T, KHELM>), g, kBlock, st, lgn, u, f, c0, c1, (T)h2, (T)ih2, (T)rho, color);
     else
         GR_LAUNCH((k_sweep<T, KPSI>), g, kBlock, st, lgn, u, f, c0, c1, (T)h2, (T)ih2, (T)rho, color);
+}
+
+void sweep_black_from_r(int n, float *e, const float *r, double h2, cudaStream_t st, int rev)
+{
+    const int64_t threads = (int64_t)n * n * n / 8;
+    GR_LAUNCH((k_sweep4<KPOISSON, true>), wave_grid(k_sweep4<KPOISSON, true>, threads), kBlock, st, log2i(n), e, r,
+              (const float *)nullptr, (float)h2, 1, rev);
 }
 
 template <typename T>
