@@ -163,15 +163,46 @@ __device__ __forceinline__ double recip64(double x)
     return fma(r, fma(-x, r, 1.0), r);
 }
 
-// the end of a reducing kernel, by every thread of the block, after thread 0
-// wrote the block's partials
+// Sums of a and b over the warp's lanes: lane 0 returns a's, lane 16 b's.  The lower half goes on with a
+// and the upper with b: five FP64 additions a warp instead of ten, each of which holds the FP64 pipe
+// for 16 cycles.
+__device__ __forceinline__ double warp_sum2(double a, double b)
+{
+    const bool up = (threadIdx.x & 16) != 0;
+    const double o = __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+    double v = (up ? b : a) + o;
+#pragma unroll
+    for (int k = 8; k > 0; k >>= 1) v += __shfl_xor_sync(0xffffffffu, v, k);
+    return v;
+}
+
+// the same over the kBlock threads of a block, returned by lanes 0 and 16 of the first warp (which
+// alone continues: the others return false); s: 2 kBlock / 32 doubles
+__device__ __forceinline__ bool block_sum_pair(double a, double b, double *s, double *v)
+{
+    constexpr int W = kBlock / 32;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const double t = warp_sum2(a, b);
+    if ((l & 15) == 0) s[(l >> 4) * W + w] = t;
+    __syncthreads();
+    if (w != 0) return false;
+    double u = (l & 15) < W ? s[(l >> 4) * W + (l & 15)] : 0.0;
+#pragma unroll
+    for (int k = W / 2; k > 0; k >>= 1) u += __shfl_xor_sync(0xffffffffu, u, k);
+    *v = u;
+    return true;
+}
+
+// the end of a reducing kernel, by every thread of the block, after lanes 0 and 16 of
+// the first warp wrote the block's partials
 __device__ __forceinline__ void last_block_sum(const Sums &S)
 {
     __shared__ bool last;
-    __shared__ double la[kBlock / 32], lb[kBlock / 32];
-    if (threadIdx.x == 0) {
+    __shared__ double la[2 * (kBlock / 32)];
+    if (threadIdx.x < 32) {
         __threadfence();
-        last = atomicInc(S.ticket, gridDim.x - 1) == gridDim.x - 1;  // wraps to zero
+        __syncwarp();
+        if (threadIdx.x == 0) last = atomicInc(S.ticket, gridDim.x - 1) == gridDim.x - 1;  // wraps to zero
     }
     __syncthreads();
     if (!last) return;
@@ -182,26 +213,15 @@ __device__ __forceinline__ void last_block_sum(const Sums &S)
         a += p.x;
         b += p.y;
     }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    if (l == 0) la[w] = a, lb[w] = b;
-    __syncthreads();
-    if (w != 0) return;
-    a = l < kBlock / 32 ? la[l] : 0.0;
-    b = l < kBlock / 32 ? lb[l] : 0.0;
-    for (int o = kBlock / 64; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    if (l == 0) {
-        S.out[0] = a;
-        S.out[1] = b;
+    double v;
+    if (!block_sum_pair(a, b, la, &v)) return;
+    const double vb = __shfl_sync(0xffffffffu, v, 16);
+    if (threadIdx.x == 0) {
+        S.out[0] = v;
+        S.out[1] = vb;
         if (S.mapped) {
-            S.mapped[0] = a;
-            S.mapped[1] = b;
+            S.mapped[0] = v;
+            S.mapped[1] = vb;
             __threadfence_system();
             if (S.flag) *(volatile double *)S.flag = S.seq;
         }
@@ -212,26 +232,9 @@ __device__ __forceinline__ void last_block_sum(const Sums &S)
 // in a fixed order.
 __device__ __forceinline__ void block_sum2(double a, double b, double *out)
 {
-    __shared__ double sa[kBlock / 32], sb[kBlock / 32];
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, o);
-        b += __shfl_down_sync(0xffffffffu, b, o);
-    }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) {
-        sa[w] = a;
-        sb[w] = b;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double ta = 0.0, tb = 0.0;
-        for (int q = 0; q < kBlock / 32; q++) {
-            ta += sa[q];
-            tb += sb[q];
-        }
-        out[2 * blockIdx.x] = ta;
-        out[2 * blockIdx.x + 1] = tb;
-    }
+    __shared__ double sa[2 * (kBlock / 32)];
+    double v;
+    if (block_sum_pair(a, b, sa, &v) && (threadIdx.x & 15) == 0) out[2 * blockIdx.x + (threadIdx.x >> 4)] = v;
 }
 
 // Sums of a and b over the grid
@@ -247,8 +250,8 @@ __device__ __forceinline__ void block_sum2(double a, double b, const Sums &S)
 // noticeable share of a memory-sized kernel.
 __device__ __forceinline__ void block_sum2f(float a, float b, const Sums &S)
 {
-    double *const out = S.partials;
-    __shared__ double sa[kBlock / 32], sb[kBlock / 32];
+    constexpr int W = kBlock / 32;
+    __shared__ double sa[2 * W];
     for (int o = 16; o > 0; o >>= 1) {
         a += __shfl_down_sync(0xffffffffu, a, o);
         b += __shfl_down_sync(0xffffffffu, b, o);
@@ -256,17 +259,14 @@ __device__ __forceinline__ void block_sum2f(float a, float b, const Sums &S)
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     if (l == 0) {
         sa[w] = (double)a;
-        sb[w] = (double)b;
+        sa[W + w] = (double)b;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double ta = 0.0, tb = 0.0;
-        for (int q = 0; q < kBlock / 32; q++) {
-            ta += sa[q];
-            tb += sb[q];
-        }
-        out[2 * blockIdx.x] = ta;
-        out[2 * blockIdx.x + 1] = tb;
+    if (w == 0) {
+        double u = (l & 15) < W ? sa[(l >> 4) * W + (l & 15)] : 0.0;
+#pragma unroll
+        for (int k = W / 2; k > 0; k >>= 1) u += __shfl_xor_sync(0xffffffffu, u, k);
+        if ((l & 15) == 0) S.partials[2 * blockIdx.x + (l >> 4)] = u;
     }
     last_block_sum(S);
 }
