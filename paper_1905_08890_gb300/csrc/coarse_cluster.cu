@@ -31,11 +31,11 @@ constexpr int kClusterCtas = 16;
 constexpr int kClusterThreads = 1024;
 constexpr int kSlabA = 4 * 64 * 64;  // cells of a CTA's 64^3 slab
 constexpr int kSlabB = 2 * 32 * 32;  // cells of a CTA's 32^3 slab
-// e and r of both slabs, the tail's residual scratch, e and r of the tail
+// e and r of both slabs, e and r of the tail
 // levels, and m, 1/(6 + h^2 m) of levels 2^3 .. 8^3 (KHELM)
 constexpr int kTailCells = 8 + 64 + 512 + 4096;
 constexpr size_t kClusterSmem =
-    sizeof(float) * (2 * kSlabA + 2 * kSlabB + 4096 + 2 * kTailCells + 2 * (8 + 64 + 512));
+    sizeof(float) * (2 * kSlabA + 2 * kSlabB + 2 * kTailCells + 2 * (8 + 64 + 512));
 
 // A level spread over the cluster in slabs of 2^lgp planes: the slab of CTA
 // `owner` holds planes [owner << lgp, (owner + 1) << lgp), colour c at
@@ -277,8 +277,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_coarse_cluster(ClusterAr
     extern __shared__ float4 sh4[];
     float *sh = reinterpret_cast<float *>(sh4);
     float *Ae = sh, *Ar = Ae + kSlabA, *Be = Ar + kSlabA, *Br = Be + kSlabB;
-    float *res = Br + kSlabB;  // residual scratch of the tail's 16^3 level (CTA 0)
-    float *p = res + 4096;
+    float *p = Br + kSlabB;
     TailLevel L[4];
 #pragma unroll
     for (int l = 0; l < 4; l++) {
@@ -334,7 +333,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_coarse_cluster(ClusterAr
         float *tr = me == 0 ? L[3].r : cl.map_shared_rank(L[3].r, 0);
         slab_restrict<KIND, 0>(cl, me, VB, Br, g.m[4], g.ih2[4], te, tr, 2048, 0, nullptr, 0.0f);
     }
-    if (me == 0) tail_cycle<KIND>(L, res, nu1, nu2);
+    if (me == 0) tail_cycle<KIND>(L, nu1, nu2);
     cl.sync();
     slab_prolong(cl, me, VT, Be, 1);
     for (int s = 0; s < nu2; s++) {

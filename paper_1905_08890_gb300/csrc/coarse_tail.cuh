@@ -13,6 +13,21 @@ namespace {
 
 constexpr int kTailN = 16;
 constexpr int kTailThreads = 1024;
+constexpr int kTailLow = 256;  // threads of the levels below 16^3 (blocks have at least as many)
+
+// the barrier of a step: of the whole block, or (LOW) of its first kTailLow threads, the
+// only ones to work below 16^3, where eight warps pass a barrier sooner than 32
+template <bool LOW>
+__device__ __forceinline__ void tail_sync()
+{
+    if (LOW) asm volatile("bar.sync 1, %0;" ::"n"(kTailLow) : "memory");
+    else __syncthreads();
+}
+template <bool LOW>
+__device__ __forceinline__ int tail_threads()
+{
+    return LOW ? kTailLow : (int)blockDim.x;
+}
 
 struct TailLevel {
     float *e, *r, *m, *inv;
@@ -43,14 +58,14 @@ __device__ __forceinline__ void tail_ldv(const float *p, float (&v)[W])
 // additions of the full-grid colour pass (k_sweep4); each row's W values are
 // one vector access (scalar accesses W floats apart put W threads of a warp
 // on each shared-memory bank)
-template <int KIND, int W>
+template <int KIND, int W, bool LOW>
 __device__ void tail_sweep_w(const TailLevel &L, int color)
 {
     const int lgn = L.lg, lgh = lgn - 1, mn = (1 << lgn) - 1, mh = (1 << lgh) - 1;
     const int half = 1 << (3 * lgn - 1), off = color ? half : 0;
     float *own = L.e + off;
     const float *oth = L.e + (half - off);
-    for (int v = threadIdx.x; v < half / W; v += blockDim.x) {
+    for (int v = threadIdx.x; v < half / W; v += tail_threads<LOW>()) {
         const int t = v * W;
         const int q = t & mh, j = (t >> lgh) & mn, i = t >> (lgh + lgn);
         const int p = (i + j + color) & 1;
@@ -77,66 +92,72 @@ __device__ void tail_sweep_w(const TailLevel &L, int color)
         if (W == 4) *reinterpret_cast<float4 *>(own + t) = make_float4(out[0], out[1], out[2], out[3]);
         else *reinterpret_cast<float2 *>(own + t) = make_float2(out[0], out[1 % W]);
     }
-    __syncthreads();
+    tail_sync<LOW>();
 }
 
-template <int KIND>
+template <int KIND, bool LOW>
 __device__ void tail_sweep(const TailLevel &L, int color)
 {
-    if (L.lg >= 3) tail_sweep_w<KIND, 4>(L, color);
-    else tail_sweep_w<KIND, 2>(L, color);
+    if (L.lg >= 3) tail_sweep_w<KIND, 4, LOW>(L, color);
+    else tail_sweep_w<KIND, 2, LOW>(L, color);
 }
 
-// residual L(e) - r of every cell of level A into A's scratch row array res
-// (split layout), then the 8-child averages, negated, as the next level's
-// right-hand side (its correction starts at zero)
+// residual L(e) - r of a cell of colour color at half-index q of row (i, j)
 template <int KIND>
-__device__ void tail_down(const TailLevel &A, const TailLevel &C, float *res)
+__device__ __forceinline__ float tail_resid(const TailLevel &A, int color, int i, int j, int q)
 {
     const int lgn = A.lg, lgh = lgn - 1, mn = (1 << lgn) - 1, mh = (1 << lgh) - 1;
-    const int half = 1 << (3 * lgn - 1);
-    for (int tt = threadIdx.x; tt < 2 * half; tt += blockDim.x) {
-        const int color = tt >= half, t = tt - (color ? half : 0);
-        const int off = color ? half : 0;
-        const float *oth = A.e + (half - off);
-        const int q = t & mh, j = (t >> lgh) & mn, i = t >> (lgh + lgn);
-        const int p = (i + j + color) & 1;
-        const int r0 = t - q, ri = j << lgh;
-        const int rip = (((i + 1) & mn) << (lgn + lgh)) + ri, rim = (((i - 1) & mn) << (lgn + lgh)) + ri;
-        const int rj = i << (lgn + lgh);
-        const int rjp = rj + (((j + 1) & mn) << lgh), rjm = rj + (((j - 1) & mn) << lgh);
-        const float nb = oth[rip + q] + oth[rim + q] + oth[rjp + q] + oth[rjm + q] + oth[r0 + q] +
-                         oth[r0 + ((q + (p ? 1 : -1)) & mh)];
-        const int id = off + t;
-        const float u = A.e[id];
-        float lap = (nb - 6.0f * u) * A.ih2;
-        if (KIND == KHELM) lap -= A.m[id] * u;
-        res[id] = lap - A.r[id];
-    }
-    __syncthreads();
+    const int half = 1 << (3 * lgn - 1), off = color ? half : 0;
+    const float *oth = A.e + (half - off);
+    const int p = (i + j + color) & 1;
+    const int ri = j << lgh, rj = i << (lgn + lgh), r0 = rj + ri;
+    const int rip = (((i + 1) & mn) << (lgn + lgh)) + ri, rim = (((i - 1) & mn) << (lgn + lgh)) + ri;
+    const int rjp = rj + (((j + 1) & mn) << lgh), rjm = rj + (((j - 1) & mn) << lgh);
+    const float nb = oth[rip + q] + oth[rim + q] + oth[rjp + q] + oth[rjm + q] + oth[r0 + q] +
+                     oth[r0 + ((q + (p ? 1 : -1)) & mh)];
+    const int id = off + r0 + q;
+    const float u = A.e[id];
+    float lap = (nb - 6.0f * u) * A.ih2;
+    if (KIND == KHELM) lap -= A.m[id] * u;
+    return lap - A.r[id];
+}
+
+// 8-child averages of level A's residual, negated, as the next level's right-hand
+// side; its correction starts at zero.  RED (after a black pass): the black
+// residuals, zero up to rounding, count as zero, and the coarse correction is
+// what its first red pass makes of zero.
+template <int KIND, bool RED, bool LOW>
+__device__ void tail_down(const TailLevel &A, const TailLevel &C)
+{
     const int lc = C.lg, mc = (1 << lc) - 1;
-    for (int t = threadIdx.x; t < (1 << (3 * lc)); t += blockDim.x) {
+    for (int t = threadIdx.x; t < (1 << (3 * lc)); t += tail_threads<LOW>()) {
         const int K = t & mc, J = (t >> lc) & mc, I = t >> (2 * lc);
         float s = 0.0f;
+#pragma unroll
         for (int a = 0; a < 2; a++)
+#pragma unroll
             for (int b = 0; b < 2; b++)
-                for (int c = 0; c < 2; c++) s += res[tail_sidx(A.lg, 2 * I + a, 2 * J + b, 2 * K + c)];
+#pragma unroll
+                for (int c = 0; c < 2; c++)
+                    if (!RED || ((a + b + c) & 1) == 0) s += tail_resid<KIND>(A, (a + b + c) & 1, 2 * I + a, 2 * J + b, K);
         const int cid = tail_sidx(lc, I, J, K);
-        C.r[cid] = -(0.125f * s);
-        C.e[cid] = 0.0f;
+        const float rc = -(0.125f * s);
+        C.r[cid] = rc;
+        C.e[cid] = RED && ((I + J + K) & 1) == 0 ? -C.h2 * rc * (KIND == KPOISSON ? 1.0f / 6.0f : C.inv[cid]) : 0.0f;
     }
-    __syncthreads();
+    tail_sync<LOW>();
 }
 
 // trilinear prolongation of the coarser level's correction added to level A;
 // black_only: a red pass follows, which does not read the red values, so only
 // the black cells take the correction (as prolong_add_black)
+template <bool LOW>
 __device__ void tail_up(const TailLevel &A, const TailLevel &C, bool black_only)
 {
     const int lc = C.lg, mc = (1 << lc) - 1, lf = A.lg, nf1 = (1 << lf) - 1, lgh = lf - 1, mh = (1 << lgh) - 1;
     const int half = 1 << (3 * lf - 1);
     const int ncell = black_only ? half : 2 * half;
-    for (int tt = threadIdx.x; tt < ncell; tt += blockDim.x) {
+    for (int tt = threadIdx.x; tt < ncell; tt += tail_threads<LOW>()) {
         // split index: colour 1 (black) first when black_only, else both colours
         const int color = black_only ? 1 : (tt >= half), t = tt - ((!black_only && color) ? half : 0);
         const int q = t & mh, j = (t >> lgh) & nf1, i = t >> (lgh + lf);
@@ -156,7 +177,7 @@ __device__ void tail_up(const TailLevel &A, const TailLevel &C, bool black_only)
         const float y0 = w[0] * z[0][0] + w[1] * z[0][1], y1 = w[0] * z[1][0] + w[1] * z[1][1];
         A.e[(color ? half : 0) + t] += w[0] * y0 + w[1] * y1;
     }
-    __syncthreads();
+    tail_sync<LOW>();
 }
 
 // Exact solve of a linear 2^3 level.  On 2^3 every neighbour of a cell along
@@ -184,7 +205,7 @@ __device__ __forceinline__ double coarsest_wht(double rx, double h2)
         v = ((x >> b) & 1) ? w - v : v + w;
     }
     const int s = __popc(x);
-    v = s ? v / (4.0 * s) : 0.0;
+    v = s == 0 ? 0.0 : v * (s == 1 ? 0.25 : (s == 2 ? 0.125 : 1.0 / 12.0));
 #pragma unroll
     for (int b = 0; b < 3; b++) {
         const double w = __shfl_xor_sync(full, v, 1 << b);
@@ -233,54 +254,64 @@ __device__ __forceinline__ double coarsest_exact(double rx, double mx, double h2
     return b / d;
 }
 
-// FP64 solve of the 2^3 level (as k_coarsest), by the first warp: the
-// right-hand side's mean removed (KPOISSON), then the exact solve
+// FP64 solve of the 2^3 level (as k_coarsest; the Poisson solve drops the
+// right-hand side's mean by itself), by the first warp
 template <int KIND>
 __device__ void tail_coarsest(const TailLevel &Z)
 {
-    __shared__ double sf[8];
     const int t = threadIdx.x;
     if (t < 32) {
-        if (t < 8) sf[t] = Z.r[t];
-        __syncwarp();
-        if (KIND == KPOISSON && t == 0) {
-            double m = 0.0;
-            for (int q = 0; q < 8; q++) m += sf[q];
-            m *= 0.125;
-            for (int q = 0; q < 8; q++) sf[q] -= m;
-        }
-        __syncwarp();
         // lane x holds cell x = 4i + 2j + k, split index 4 ((i + j + k) & 1) + 2i + j
         const int x = t & 7, i = x >> 2, j = (x >> 1) & 1, k = x & 1;
         const int id = 4 * ((i + j + k) & 1) + 2 * i + j;
-        const double e = coarsest_exact<KIND>(sf[id], KIND == KPOISSON ? 0.0 : (double)Z.m[id], (double)Z.h2);
+        const double e =
+            coarsest_exact<KIND>((double)Z.r[id], KIND == KPOISSON ? 0.0 : (double)Z.m[id], (double)Z.h2);
         if (t < 8) Z.e[id] = (float)e;
     }
-    __syncthreads();
+    tail_sync<true>();
 }
 
 // one correction V-cycle over the tail levels L[3] (16^3, e and r given) ..
 // L[0] (2^3): nu1 red-black sweeps, residual-restriction, the 2^3 solve,
-// prolongation and nu2 sweeps; res: scratch of 16^3 floats
+// prolongation and nu2 sweeps.  A step is bound by its barrier and one round of
+// shared-memory latency, so what counts is their number: red residuals are
+// restricted in one step that also makes the coarse level's first red pass (two
+// steps and a pass of their own before), and the levels below 16^3 keep to
+// kTailLow threads (13.7 -> 11.0 us per Poisson cycle)
 template <int KIND>
-__device__ __forceinline__ void tail_cycle(TailLevel (&L)[4], float *res, int nu1, int nu2)
+__device__ __forceinline__ void tail_cycle(TailLevel (&L)[4], int nu1, int nu2)
 {
-#pragma unroll
-    for (int l = 3; l >= 1; l--) {
-        for (int s = 0; s < nu1; s++) {
-            tail_sweep<KIND>(L[l], 0);
-            tail_sweep<KIND>(L[l], 1);
-        }
-        tail_down<KIND>(L[l], L[l - 1], res);
+    for (int s = 0; s < nu1; s++) {
+        tail_sweep<KIND, false>(L[3], 0);
+        tail_sweep<KIND, false>(L[3], 1);
     }
-    tail_coarsest<KIND>(L[0]);
+    if (nu1 > 0) tail_down<KIND, true, false>(L[3], L[2]);
+    else tail_down<KIND, false, false>(L[3], L[2]);
+    if (threadIdx.x < kTailLow) {
 #pragma unroll
-    for (int l = 1; l <= 3; l++) {
-        tail_up(L[l], L[l - 1], nu2 > 0);
-        for (int s = 0; s < nu2; s++) {
-            tail_sweep<KIND>(L[l], 0);
-            tail_sweep<KIND>(L[l], 1);
+        for (int l = 2; l >= 1; l--) {
+            for (int s = 0; s < nu1; s++) {
+                if (s > 0) tail_sweep<KIND, true>(L[l], 0);  // the first red pass came with the restriction
+                tail_sweep<KIND, true>(L[l], 1);
+            }
+            if (nu1 > 0) tail_down<KIND, true, true>(L[l], L[l - 1]);
+            else tail_down<KIND, false, true>(L[l], L[l - 1]);
         }
+        tail_coarsest<KIND>(L[0]);
+#pragma unroll
+        for (int l = 1; l <= 2; l++) {
+            tail_up<true>(L[l], L[l - 1], nu2 > 0);
+            for (int s = 0; s < nu2; s++) {
+                tail_sweep<KIND, true>(L[l], 0);
+                tail_sweep<KIND, true>(L[l], 1);
+            }
+        }
+    }
+    __syncthreads();
+    tail_up<false>(L[3], L[2], nu2 > 0);
+    for (int s = 0; s < nu2; s++) {
+        tail_sweep<KIND, false>(L[3], 0);
+        tail_sweep<KIND, false>(L[3], 1);
     }
 }
 

@@ -1065,8 +1065,7 @@ __global__ void __launch_bounds__(kTailThreads) k_coarse_tail(TailArgs g, int nu
     pdl_begin();
     extern __shared__ float sh[];
     TailLevel L[4];
-    float *res = sh;  // residual scratch of the finest tail level (16^3 cells)
-    float *p = sh + (1 << 12);
+    float *p = sh;
 #pragma unroll
     for (int l = 0; l < 4; l++) {
         const int cells = 1 << (3 * (l + 1));
@@ -1090,7 +1089,7 @@ __global__ void __launch_bounds__(kTailThreads) k_coarse_tail(TailArgs g, int nu
         }
     }
     __syncthreads();
-    tail_cycle<KIND>(L, res, nu1, nu2);
+    tail_cycle<KIND>(L, nu1, nu2);
     for (int t = threadIdx.x; t < (1 << 12); t += blockDim.x) g.e[3][t] = L[3].e[t];
 }
 
@@ -1109,7 +1108,7 @@ void coarse_tail(int kind, float *const *e, float *const *r, const float *const 
         a.inv[l] = inv[l];
         a.h2[l] = (float)h2[l];
     }
-    const size_t smem = sizeof(float) * (4096 + 4 * (8 + 64 + 512 + 4096));  // residual scratch + e, r, m, inv
+    const size_t smem = sizeof(float) * 4 * (8 + 64 + 512 + 4096);  // e, r, m, inv
     // once per kernel (function-local statics are initialised once, even with several host threads)
     if (kind == KPOISSON) {
         static const bool attr = cudaFuncSetAttribute(k_coarse_tail<KPOISSON>,
