@@ -242,7 +242,7 @@ __device__ __forceinline__ double coarsest_exact(double rx, double mx, double h2
 #pragma unroll
         for (int k = p + 1; k < 8; k++) row[k] = __shfl_sync(full, a[k], src);
         if (x != p) {
-            const double f = a[p] / piv;
+            const double f = a[p] * recip64(piv);
 #pragma unroll
             for (int k = p + 1; k < 8; k++) a[k] = fma(-f, row[k], a[k]);
             b = fma(-f, bp, b);
@@ -251,7 +251,7 @@ __device__ __forceinline__ double coarsest_exact(double rx, double mx, double h2
     double d = a[0];
 #pragma unroll
     for (int y = 1; y < 8; y++) d = y == x ? a[y] : d;
-    return b / d;
+    return b * recip64(d);
 }
 
 // FP64 solve of the 2^3 level (as k_coarsest; the Poisson solve drops the
