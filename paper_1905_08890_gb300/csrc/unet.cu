@@ -132,15 +132,15 @@ void forward(gr_net *net, const gr_sources *s, double rho, double vrms)
     cv(6);
     cv(7);
     gr::upsample(net->act[T_E3B], 128, net->lg0 - 3, net->act[T_CAT2], 192, st);
-    gr::copy_slice(net->act[T_E2B], 64, 64, 0, net->act[T_CAT2], 192, 128, nvox(net, 2), 0, st);
+    gr::copy_slice(net->act[T_E2B], 64, 64, 0, net->act[T_CAT2], 192, 128, nvox(net, 2), st);
     cv(8);
     cv(9);
     gr::upsample(net->act[T_D2B], 64, net->lg0 - 2, net->act[T_CAT1], 96, st);
-    gr::copy_slice(net->act[T_E1B], 32, 32, 0, net->act[T_CAT1], 96, 64, nvox(net, 1), 0, st);
+    gr::copy_slice(net->act[T_E1B], 32, 32, 0, net->act[T_CAT1], 96, 64, nvox(net, 1), st);
     cv(10);
     cv(11);
     gr::upsample(net->act[T_D1B], 32, net->lg0 - 1, net->act[T_CAT0], 48, st);
-    gr::copy_slice(net->act[T_E0B], 16, 16, 0, net->act[T_CAT0], 48, 32, nv0, 0, st);
+    gr::copy_slice(net->act[T_E0B], 16, 16, 0, net->act[T_CAT0], 48, 32, nv0, st);
     cv(12);
     cv(13);
     gr::head(net->act[T_D0B], net->params + net->head_w, net->params + net->head_b, nv0, net->out, st);
@@ -162,39 +162,30 @@ void backward(gr_net *net)
         const Conv &c = net->conv[k];
         const int lg = net->lg0 - c.lev;
         const int in = kConvIO[k][0], outt = kConvIO[k][1];
-        gr::conv3d_wgrad(net->act[in], c.cin, net->grad[outt], c.cout, lg, net->grads + c.w, st);
-        gr::bias_grad(net->grad[outt], c.cout, nvox(net, c.lev), net->grads + c.b, st);
+        gr::conv3d_wgrad(net->act[in], c.cin, net->grad[outt], c.cout, lg, net->grads + c.w,
+                         net->grads + c.b, st);
         if (dgrad_mode >= 0)
             gr::conv3d(net->grad[outt], c.cout, net->wt + c.wb, nullptr, c.cin, lg, dgrad_mode,
                        dgrad_mode == CONV_MASK ? net->act[in] : nullptr, net->grad[in], st);
     };
     back(13, CONV_MASK);   // -> grad d0a (through d0a's ReLU)
     back(12, CONV_PLAIN);  // -> grad cat0
-    gr::upsample_back(net->grad[T_CAT0], 32, 48, net->lg0 - 1, net->grad[T_D1B], st);
-    gr::relu_mask(net->grad[T_D1B], net->act[T_D1B], nvox(net, 1) * 32, st);
-    gr::copy_slice(net->grad[T_CAT0], 16, 48, 32, net->grad[T_E0B], 16, 0, nv0, 0, st);
+    gr::upsample_back(net->grad[T_CAT0], 32, 48, net->lg0 - 1, net->act[T_D1B], net->grad[T_D1B], st);
     back(11, CONV_MASK);
     back(10, CONV_PLAIN);
-    gr::upsample_back(net->grad[T_CAT1], 64, 96, net->lg0 - 2, net->grad[T_D2B], st);
-    gr::relu_mask(net->grad[T_D2B], net->act[T_D2B], nvox(net, 2) * 64, st);
-    gr::copy_slice(net->grad[T_CAT1], 32, 96, 64, net->grad[T_E1B], 32, 0, nvox(net, 1), 0, st);
+    gr::upsample_back(net->grad[T_CAT1], 64, 96, net->lg0 - 2, net->act[T_D2B], net->grad[T_D2B], st);
     back(9, CONV_MASK);
     back(8, CONV_PLAIN);
-    gr::upsample_back(net->grad[T_CAT2], 128, 192, net->lg0 - 3, net->grad[T_E3B], st);
-    gr::relu_mask(net->grad[T_E3B], net->act[T_E3B], nvox(net, 3) * 128, st);
-    gr::copy_slice(net->grad[T_CAT2], 64, 192, 128, net->grad[T_E2B], 64, 0, nvox(net, 2), 0, st);
+    gr::upsample_back(net->grad[T_CAT2], 128, 192, net->lg0 - 3, net->act[T_E3B], net->grad[T_E3B], st);
     back(7, CONV_MASK);
     back(6, CONV_PLAIN);  // -> grad p3
-    gr::pool_back(net->grad[T_P3], 64, net->lg0 - 2, net->grad[T_E2B], 64, 1, st);
-    gr::relu_mask(net->grad[T_E2B], net->act[T_E2B], nvox(net, 2) * 64, st);
+    gr::skip_back(net->grad[T_P3], 64, net->lg0 - 2, net->grad[T_CAT2], 192, 128, net->act[T_E2B], net->grad[T_E2B], st);
     back(5, CONV_MASK);
     back(4, CONV_PLAIN);
-    gr::pool_back(net->grad[T_P2], 32, net->lg0 - 1, net->grad[T_E1B], 32, 1, st);
-    gr::relu_mask(net->grad[T_E1B], net->act[T_E1B], nvox(net, 1) * 32, st);
+    gr::skip_back(net->grad[T_P2], 32, net->lg0 - 1, net->grad[T_CAT1], 96, 64, net->act[T_E1B], net->grad[T_E1B], st);
     back(3, CONV_MASK);
     back(2, CONV_PLAIN);
-    gr::pool_back(net->grad[T_P1], 16, net->lg0, net->grad[T_E0B], 16, 1, st);
-    gr::relu_mask(net->grad[T_E0B], net->act[T_E0B], nv0 * 16, st);
+    gr::skip_back(net->grad[T_P1], 16, net->lg0, net->grad[T_CAT0], 48, 32, net->act[T_E0B], net->grad[T_E0B], st);
     back(1, CONV_MASK);
     back(0, -1);
 }

@@ -27,17 +27,17 @@ bool conv3d_tc_fits(int cin, int cout, int lg);
 void conv3d_tc(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, const float *bias, int cout, int mode,
                const __nv_bfloat16 *mask, __nv_bfloat16 *y, cudaStream_t st);
 int conv3d_tc_error(cudaStream_t st);
-void conv3d_wgrad(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *dy, int cout, int lg, float *dw,
+// weight and bias gradients, added to dw and db
+void conv3d_wgrad(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *dy, int cout, int lg, float *dw, float *db,
                   cudaStream_t st);
-void bias_grad(const __nv_bfloat16 *dy, int c, int64_t nv, float *db, cudaStream_t st);
 void pool(const __nv_bfloat16 *x, int c, int cstride, int lgf, __nv_bfloat16 *y, cudaStream_t st);
-void pool_back(const __nv_bfloat16 *dy, int c, int lgf, __nv_bfloat16 *dx, int cstride, int accumulate,
-               cudaStream_t st);
+void skip_back(const __nv_bfloat16 *dy, int c, int lgf, const __nv_bfloat16 *skip, int ss, int soff,
+               const __nv_bfloat16 *act, __nv_bfloat16 *dx, cudaStream_t st);
 void upsample(const __nv_bfloat16 *x, int c, int lgc, __nv_bfloat16 *y, int cstride, cudaStream_t st);
-void upsample_back(const __nv_bfloat16 *dy, int c, int cstride, int lgc, __nv_bfloat16 *dx, cudaStream_t st);
+void upsample_back(const __nv_bfloat16 *dy, int c, int cstride, int lgc, const __nv_bfloat16 *act, __nv_bfloat16 *dx,
+                   cudaStream_t st);
 void copy_slice(const __nv_bfloat16 *x, int c, int xs, int xoff, __nv_bfloat16 *y, int ys, int yoff, int64_t nv,
-                int accumulate, cudaStream_t st);
-void relu_mask(__nv_bfloat16 *g, const __nv_bfloat16 *a, int64_t total, cudaStream_t st);
+                cudaStream_t st);
 void net_input(const double *s0, const double *sx, const double *sy, const double *sz, int64_t nv, float inv_rho,
                float inv_rv, const float *in_mean, const float *in_std, __nv_bfloat16 *x, cudaStream_t st);
 void head(const __nv_bfloat16 *a, const float *W, const float *b, int64_t nv, float *out, cudaStream_t st);

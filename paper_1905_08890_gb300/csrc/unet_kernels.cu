@@ -252,12 +252,13 @@ void launch_conv3d(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, cons
 // dy and of x with its halo are staged in shared memory, one box ahead; both
 // operands are read transposed (ldmatrix .trans) from the voxel rows, A once
 // for a warp's three taps.  The taps' sums stay in registers over the block's
-// boxes and end in one FP32 atomic per weight.  (One tap per block with
+// boxes and end in one FP32 atomic per weight.  The blocks of the first 16 input
+// channels also sum dy itself, the bias's gradient (4.4 us a layer as a launch of its own).  (One tap per block with
 // two-byte gathers took 957 us over the layers at 64^3; these take 304.)
 constexpr int kWgWarps = 9, kWgBox = 8;  // boxes of 2^8 voxels (or the grid)
 __global__ void __launch_bounds__(32 * kWgWarps)
     k_conv3d_wgrad(const __nv_bfloat16 *__restrict__ x, int cin, const __nv_bfloat16 *__restrict__ dy, int cout, Box bx,
-                   int nbox, float *__restrict__ dw)
+                   int nbox, float *__restrict__ dw, float *__restrict__ db)
 {
     pdl_begin();
     extern __shared__ __align__(128) unsigned char csm[];
@@ -288,6 +289,10 @@ __global__ void __launch_bounds__(32 * kWgWarps)
     // 8..15; B (voxels x ci): voxels 0..7 and 8..15 of ci 0..7, then of ci 8..15
     const int arow = (lane & 7) + ((lane >> 4) << 3), ahalf = (lane >> 3) & 1;
     const int brow = (lane & 7) + (((lane >> 3) & 1) << 3), bhalf = lane >> 4;
+    // bias: thread t < 256 sums channel t mod 16 over every 16th voxel
+    const bool bias = ci0 == 0 && threadIdx.x < 256;
+    const int bc = threadIdx.x & 15;
+    float bsum = 0.0f;
     if (first < last) load(first, base);
     for (int b = first, k = 0; b < last; b++, k ^= 1) {
         const uint32_t buf = base + (k ? stage : 0u);
@@ -311,9 +316,25 @@ __global__ void __launch_bounds__(32 * kWgWarps)
                 mma_bf16(acc[j][1], af, b1);
             }
         }
+        if (bias) {
+            const unsigned char *dyb = csm + (buf - base) + 32 * halo + 2 * (bc & 7);
+            for (int q = threadIdx.x >> 4; q < nv; q += 16)
+                bsum += __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(dyb + row_half(q, bc >> 3)));
+        }
         __syncthreads();  // before the next box's copies overwrite this buffer
     }
     if (first >= last) return;
+    if (ci0 == 0) {
+        float *sb = reinterpret_cast<float *>(csm);
+        bsum += __shfl_xor_sync(0xffffffffu, bsum, 16);
+        if (threadIdx.x < 256 && lane < 16) sb[16 * warp + lane] = bsum;
+        __syncthreads();
+        if (threadIdx.x < 16) {
+            float v = 0.0f;
+            for (int k = 0; k < 8; k++) v += sb[16 * k + threadIdx.x];
+            atomicAdd(db + co0 + threadIdx.x, v);
+        }
+    }
     // acc[j][n][0..1]: co g, ci 8 n + 2 t (+ 1); [2..3]: co g + 8
 #pragma unroll
     for (int j = 0; j < 3; j++)
@@ -323,27 +344,6 @@ __global__ void __launch_bounds__(32 * kWgWarps)
             for (int r = 0; r < 4; r++)
                 atomicAdd(dw + ((size_t)(3 * warp + j) * cout + co0 + g + 8 * (r >> 1)) * cin + ci0 + 8 * n + 2 * t + (r & 1),
                           acc[j][n][r]);
-}
-
-// ---------------------------------------------------------------- small layers
-// per-channel sum over voxels of dy (bias gradient).  The grid stride
-// (kBiasBlocks * 256 = 2^11 * 57) is a multiple of every channel count of the
-// network (16 ... 192 = 2^6 * 3), so each thread always meets one channel.
-constexpr int kBiasBlocks = 456;
-__global__ void __launch_bounds__(256)
-    k_bias_grad(const __nv_bfloat16 *__restrict__ dy, int c, int64_t nv, float *__restrict__ db)
-{
-    pdl_begin();
-    extern __shared__ float sbuf[];
-    for (int k = threadIdx.x; k < c; k += blockDim.x) sbuf[k] = 0.0f;
-    __syncthreads();
-    const int64_t total = nv * c;
-    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    float s = 0.0f;
-    for (int64_t e = first; e < total; e += (int64_t)gridDim.x * blockDim.x) s += __bfloat162float(dy[e]);
-    atomicAdd(&sbuf[first % c], s);
-    __syncthreads();
-    for (int k = threadIdx.x; k < c; k += blockDim.x) atomicAdd(db + k, sbuf[k]);
 }
 
 // 2^3 average pooling, channels-last; fine extent 2^lgf
@@ -364,25 +364,6 @@ __global__ void k_pool(const __nv_bfloat16 *__restrict__ x, int c, int cstride, 
                     s += __bfloat162float(x[(size_t)v * cstride + ch]);
                 }
         y[e] = __float2bfloat16(0.125f * s);
-    }
-}
-
-// adjoint of k_pool: dx[v][ch] (+)= dy[parent][ch] / 8 (into a strided slice)
-__global__ void k_pool_back(const __nv_bfloat16 *__restrict__ dy, int c, int lgf, __nv_bfloat16 *__restrict__ dx,
-                            int cstride, int accumulate)
-{
-    pdl_begin();
-    const int mf = (1 << lgf) - 1, lgc = lgf - 1;
-    const int64_t total = ((int64_t)1 << (3 * lgf)) * c;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int ch = (int)(e % c);
-        const int v = (int)(e / c);
-        const int k = v & mf, j = (v >> lgf) & mf, i = v >> (2 * lgf);
-        const int V = ((((i >> 1) << lgc) + (j >> 1)) << lgc) + (k >> 1);
-        float g = 0.125f * __bfloat162float(dy[(size_t)V * c + ch]);
-        __nv_bfloat16 *o = dx + (size_t)v * cstride + ch;
-        if (accumulate) g += __bfloat162float(*o);
-        *o = __float2bfloat16(g);
     }
 }
 
@@ -416,52 +397,17 @@ __global__ void k_upsample(const __nv_bfloat16 *__restrict__ x, int c, int lgc, 
     }
 }
 
-// adjoint of k_upsample: per axis coarse J gathers fine 2J-1 (1/4), 2J (3/4),
-// 2J+1 (3/4), 2J+2 (1/4); dy read from channels [0, c) of stride cstride
-__global__ void k_upsample_back(const __nv_bfloat16 *__restrict__ dy, int c, int cstride, int lgc,
-                                __nv_bfloat16 *__restrict__ dx)
-{
-    pdl_begin();
-    const int lgf = lgc + 1, mf = (1 << lgf) - 1, mc = (1 << lgc) - 1;
-    const int64_t total = ((int64_t)1 << (3 * lgc)) * c;
-    const float wt[4] = {0.25f, 0.75f, 0.75f, 0.25f};
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int ch = (int)(e % c);
-        const int V = (int)(e / c);
-        const int K = V & mc, J = (V >> lgc) & mc, I = V >> (2 * lgc);
-        float s = 0.0f;
-        for (int a = 0; a < 4; a++)
-            for (int b = 0; b < 4; b++)
-                for (int q = 0; q < 4; q++) {
-                    const int i = (2 * I - 1 + a) & mf, j = (2 * J - 1 + b) & mf, k = (2 * K - 1 + q) & mf;
-                    s += wt[a] * wt[b] * wt[q] * __bfloat162float(dy[(size_t)((((i << lgf) + j) << lgf) + k) * cstride + ch]);
-                }
-        dx[e] = __float2bfloat16(s);
-    }
-}
-
-// y[v][off + ch] = x[v][ch] (copy into a channel slice); back: the reverse
+// y[v][yoff + ch] = x[v][xoff + ch] (copy into a channel slice)
 __global__ void k_copy_slice(const __nv_bfloat16 *__restrict__ x, int c, int xs, int xoff, __nv_bfloat16 *__restrict__ y,
-                             int ys, int yoff, int64_t nv, int accumulate)
+                             int ys, int yoff, int64_t nv)
 {
     pdl_begin();
     const int64_t total = nv * c;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int ch = (int)(e % c);
         const int64_t v = e / c;
-        float val = __bfloat162float(x[v * xs + xoff + ch]);
-        __nv_bfloat16 *o = y + v * ys + yoff + ch;
-        if (accumulate) val += __bfloat162float(*o);
-        *o = __float2bfloat16(val);
+        y[v * ys + yoff + ch] = x[v * xs + xoff + ch];
     }
-}
-
-// g *= (a > 0) elementwise (ReLU backward where the gradient was summed first)
-__global__ void k_relu_mask(__nv_bfloat16 *__restrict__ gbuf, const __nv_bfloat16 *__restrict__ a, int64_t total)
-{
-    pdl_begin();
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x)
-        if (!(__bfloat162float(a[e]) > 0.0f)) gbuf[e] = __float2bfloat16(0.0f);
 }
 
 // Eight channels per thread (c and the channel strides and offsets multiples
@@ -533,24 +479,75 @@ __global__ void __launch_bounds__(256)
     }
 }
 
+// Gradient of a level's last encoder activation act: through the skip connection
+// (channels [soff, soff + c) of the concatenation's gradient, stride ss) plus the
+// pooling's, dy / 8 of the parent, through act's ReLU
+__global__ void k_skip_back8(const __nv_bfloat16 *__restrict__ dy, int lgc8, int lgf, const __nv_bfloat16 *__restrict__ skip,
+                             int ss, int soff, const __nv_bfloat16 *__restrict__ act, __nv_bfloat16 *__restrict__ dx)
+{
+    pdl_begin();
+    const int mf = (1 << lgf) - 1, lgc = lgf - 1, c = 8 << lgc8;
+    const int64_t total = (int64_t)1 << (3 * lgf + lgc8);
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int ch = (int)(e & ((1 << lgc8) - 1)) << 3;
+        const int v = (int)(e >> lgc8);
+        const int k = v & mf, j = (v >> lgf) & mf, i = v >> (2 * lgf);
+        const int V = ((((i >> 1) << lgc) + (j >> 1)) << lgc) + (k >> 1);
+        float g[8], s[8], a[8];
+        bf8_unpack(*reinterpret_cast<const uint4 *>(dy + (size_t)V * c + ch), g);
+        bf8_unpack(*reinterpret_cast<const uint4 *>(skip + (size_t)v * ss + soff + ch), s);
+        bf8_unpack(*reinterpret_cast<const uint4 *>(act + (size_t)v * c + ch), a);
+#pragma unroll
+        for (int m = 0; m < 8; m++) g[m] = a[m] > 0.0f ? 0.125f * g[m] + s[m] : 0.0f;
+        *reinterpret_cast<uint4 *>(dx + (size_t)v * c + ch) = bf8_pack(g);
+    }
+}
+
+// adjoint of the upsampling: per axis coarse J gathers fine 2J-1 (1/4), 2J (3/4),
+// 2J+1 (3/4), 2J+2 (1/4); dy read from channels [0, c) of stride cstride; through
+// the ReLU of the activation act that was upsampled
+__global__ void k_upsample_back8(const __nv_bfloat16 *__restrict__ dy, int lgc8, int cstride, int lgc,
+                                 const __nv_bfloat16 *__restrict__ act, __nv_bfloat16 *__restrict__ dx)
+{
+    pdl_begin();
+    const int lgf = lgc + 1, mf = (1 << lgf) - 1, mc = (1 << lgc) - 1, c = 8 << lgc8;
+    const int64_t total = (int64_t)1 << (3 * lgc + lgc8);
+    const float wt[4] = {0.25f, 0.75f, 0.75f, 0.25f};
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int ch = (int)(e & ((1 << lgc8) - 1)) << 3;
+        const int V = (int)(e >> lgc8);
+        const int K = V & mc, J = (V >> lgc) & mc, I = V >> (2 * lgc);
+        float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, a8[8];
+#pragma unroll
+        for (int a = 0; a < 4; a++)
+#pragma unroll
+            for (int b = 0; b < 4; b++)
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const int i = (2 * I - 1 + a) & mf, j = (2 * J - 1 + b) & mf, k = (2 * K - 1 + q) & mf;
+                    const float w = wt[a] * wt[b] * wt[q];
+                    float g[8];
+                    bf8_unpack(*reinterpret_cast<const uint4 *>(dy + (size_t)((((i << lgf) + j) << lgf) + k) * cstride + ch), g);
+#pragma unroll
+                    for (int m = 0; m < 8; m++) s[m] += w * g[m];
+                }
+        bf8_unpack(*reinterpret_cast<const uint4 *>(act + (size_t)V * c + ch), a8);
+#pragma unroll
+        for (int m = 0; m < 8; m++) s[m] = a8[m] > 0.0f ? s[m] : 0.0f;
+        *reinterpret_cast<uint4 *>(dx + (size_t)V * c + ch) = bf8_pack(s);
+    }
+}
+
 __global__ void k_copy_slice8(const __nv_bfloat16 *__restrict__ x, int lgc8, int xs, int xoff,
-                              __nv_bfloat16 *__restrict__ y, int ys, int yoff, int nv, int accumulate)
+                              __nv_bfloat16 *__restrict__ y, int ys, int yoff, int nv)
 {
     pdl_begin();
     const int total = nv << lgc8;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
         const int ch = (e & ((1 << lgc8) - 1)) << 3;
         const int v = e >> lgc8;
-        float val[8];
-        bf8_unpack(*reinterpret_cast<const uint4 *>(x + (size_t)v * xs + xoff + ch), val);
-        uint4 *o = reinterpret_cast<uint4 *>(y + (size_t)v * ys + yoff + ch);
-        if (accumulate) {
-            float prev[8];
-            bf8_unpack(*o, prev);
-#pragma unroll
-            for (int m = 0; m < 8; m++) val[m] += prev[m];
-        }
-        *o = bf8_pack(val);
+        *reinterpret_cast<uint4 *>(y + (size_t)v * ys + yoff + ch) =
+            *reinterpret_cast<const uint4 *>(x + (size_t)v * xs + xoff + ch);
     }
 }
 
@@ -866,18 +863,20 @@ void conv3d(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, const float
         conv3d_tc(x, cin, w, bias, cout, mode, mask, y, st);
         return;
     }
-    // 256 voxels x 32 (16) channels per block where that gives every SM two blocks, else 64 voxels x
-    // 16 channels (16^3, 128 -> 128: 21 us; 8^3 at 64^3's coarsest level had 16 blocks of 62 us)
+    // 256 voxels x 32 channels per block where that gives every SM two blocks, x 16 channels down to 256
+    // blocks (32^3, 32 -> 32: 11.8 us against 18.3), else 64 voxels x 16 channels (16^3, 64 -> 128: 128
+    // blocks would take longer; 8^3 at 64^3's coarsest level had 16 blocks of 62 us)
     const int64_t nv = (int64_t)1 << (3 * lg);
-    if (lg >= 3 && (nv >> 8) * (cout / 16) >= 304) {
-        if (cout % 32 == 0) launch_conv3d<8, 2, 4>(x, cin, w, bias, cout, lg, 8, mode, mask, y, st);
+    const int64_t blocks = (nv >> 8) * (cout / 16);  // of 256 voxels x 16 channels
+    if (lg >= 3 && blocks >= 256) {
+        if (cout % 32 == 0 && blocks >= 304) launch_conv3d<8, 2, 4>(x, cin, w, bias, cout, lg, 8, mode, mask, y, st);
         else launch_conv3d<8, 2, 2>(x, cin, w, bias, cout, lg, 8, mode, mask, y, st);
     } else {
         launch_conv3d<4, 1, 2>(x, cin, w, bias, cout, lg, 6, mode, mask, y, st);
     }
 }
 
-void conv3d_wgrad(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *dy, int cout, int lg, float *dw,
+void conv3d_wgrad(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *dy, int cout, int lg, float *dw, float *db,
                   cudaStream_t st)
 {
     const int lb = 3 * lg < kWgBox ? 3 * lg : kWgBox;
@@ -891,22 +890,12 @@ void conv3d_wgrad(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *dy, int 
         cudaFuncSetAttribute(k_conv3d_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) == cudaSuccess;
     (void)attr;
     const int smem = 2 * 32 * (bx.halo() + (1 << lb));
-    GR_LAUNCH_SMEM(k_conv3d_wgrad, dim3(split, pairs), 32 * kWgWarps, smem, st, x, cin, dy, cout, bx, nbox, dw);
-}
-
-void bias_grad(const __nv_bfloat16 *dy, int c, int64_t nv, float *db, cudaStream_t st)
-{
-    GR_LAUNCH_SMEM(k_bias_grad, kBiasBlocks, 256, c * sizeof(float), st, dy, c, nv, db);
+    GR_LAUNCH_SMEM(k_conv3d_wgrad, dim3(split, pairs), 32 * kWgWarps, smem, st, x, cin, dy, cout, bx, nbox, dw, db);
 }
 
 void pool(const __nv_bfloat16 *x, int c, int cstride, int lgf, __nv_bfloat16 *y, cudaStream_t st)
 {
     GR_LAUNCH(k_pool, cdiv(((int64_t)1 << (3 * lgf - 3)) * c, 256), 256, st, x, c, cstride, lgf, y);
-}
-
-void pool_back(const __nv_bfloat16 *dy, int c, int lgf, __nv_bfloat16 *dx, int cstride, int accumulate, cudaStream_t st)
-{
-    GR_LAUNCH(k_pool_back, cdiv(((int64_t)1 << (3 * lgf)) * c, 256), 256, st, dy, c, lgf, dx, cstride, accumulate);
 }
 
 // exponent of a power of two, -1 otherwise
@@ -928,25 +917,29 @@ void upsample(const __nv_bfloat16 *x, int c, int lgc, __nv_bfloat16 *y, int cstr
     GR_LAUNCH(k_upsample, cdiv(((int64_t)1 << (3 * lgc + 3)) * c, 256), 256, st, x, c, lgc, y, cstride);
 }
 
-void upsample_back(const __nv_bfloat16 *dy, int c, int cstride, int lgc, __nv_bfloat16 *dx, cudaStream_t st)
+void skip_back(const __nv_bfloat16 *dy, int c, int lgf, const __nv_bfloat16 *skip, int ss, int soff,
+               const __nv_bfloat16 *act, __nv_bfloat16 *dx, cudaStream_t st)
 {
-    GR_LAUNCH(k_upsample_back, cdiv(((int64_t)1 << (3 * lgc)) * c, 256), 256, st, dy, c, cstride, lgc, dx);
+    const int l8 = pow2_log(c) - 3;  // every level has 16 2^l channels
+    GR_LAUNCH(k_skip_back8, cdiv((int64_t)1 << (3 * lgf + l8), 256), 256, st, dy, l8, lgf, skip, ss, soff, act, dx);
+}
+
+void upsample_back(const __nv_bfloat16 *dy, int c, int cstride, int lgc, const __nv_bfloat16 *act, __nv_bfloat16 *dx,
+                   cudaStream_t st)
+{
+    const int l8 = pow2_log(c) - 3;
+    GR_LAUNCH(k_upsample_back8, cdiv((int64_t)1 << (3 * lgc + l8), 128), 128, st, dy, l8, cstride, lgc, act, dx);
 }
 
 void copy_slice(const __nv_bfloat16 *x, int c, int xs, int xoff, __nv_bfloat16 *y, int ys, int yoff, int64_t nv,
-                int accumulate, cudaStream_t st)
+                cudaStream_t st)
 {
     const int l8 = pow2_log(c) - 3;
     if (l8 >= 0 && xs % 8 == 0 && ys % 8 == 0 && xoff % 8 == 0 && yoff % 8 == 0 && (nv << l8) < (1LL << 31)) {
-        GR_LAUNCH(k_copy_slice8, cdiv(nv << l8, 256), 256, st, x, l8, xs, xoff, y, ys, yoff, (int)nv, accumulate);
+        GR_LAUNCH(k_copy_slice8, cdiv(nv << l8, 256), 256, st, x, l8, xs, xoff, y, ys, yoff, (int)nv);
         return;
     }
-    GR_LAUNCH(k_copy_slice, cdiv(nv * c, 256), 256, st, x, c, xs, xoff, y, ys, yoff, nv, accumulate);
-}
-
-void relu_mask(__nv_bfloat16 *g, const __nv_bfloat16 *a, int64_t total, cudaStream_t st)
-{
-    GR_LAUNCH(k_relu_mask, cdiv(total, 256), 256, st, g, a, total);
+    GR_LAUNCH(k_copy_slice, cdiv(nv * c, 256), 256, st, x, c, xs, xoff, y, ys, yoff, nv);
 }
 
 void net_input(const double *s0, const double *sx, const double *sy, const double *sz, int64_t nv, float inv_rho,
