@@ -1033,7 +1033,6 @@ void to_float(int64_t cnt, const double *a, float *b, cudaStream_t st)
                                   cudaStream_t, int);                                                              \
     template void resid_restrict<T>(int, int, const T *, const T *, const T *, const T *, double, double, T *, T *, \
                                     T *, int, cudaStream_t, bool);                                                 \
-    template void prolong_add<T>(int, T *, const T *, cudaStream_t);                                               \
     template void coarsest<T>(int, T *, T *, const T *, const T *, double, double, double, cudaStream_t);           \
     template void restrict_coef<T>(int, int, const T *, const T *, T *, T *, double, cudaStream_t);                \
     template void helm_invdiag<T>(int, const T *, T *, double, cudaStream_t);                                      \
@@ -1041,6 +1040,7 @@ void to_float(int64_t cnt, const double *a, float *b, cudaStream_t st)
                                 const Sums &, double *, cudaStream_t);
 GR_INST(double)
 GR_INST(float)
+template void prolong_add<float>(int, float *, const float *, cudaStream_t);  // FP64: prolong64
 
 // ================================================================ coarse tail
 // Levels 16^3 down to 2^3 and back up of one FP32 correction V-cycle
