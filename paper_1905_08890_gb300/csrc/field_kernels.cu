@@ -185,9 +185,9 @@ __global__ void __launch_bounds__(kBlock)
 // A_ij of Eq. Aij-discrete-2 (xx yy zz xy xz yz, natural) and AA = A_ij A^ij.
 // FP64 issue is the bound, so the sums are formed on unscaled differences, in
 // units of 1/2h (r = 2 (1/h^2) / (1/2h), the second derivatives' factor in
-// those units), and scaled once: 45 operations per cell for AA and 6 more for
-// the stored A_ij, where scaling every derivative took 65.  256^3: 1.97 -> 1.42
-// ms without the stores (45 operations at the measured FP64 rate: 1.43).
+// those units), and scaled once: 48 operations per cell for AA and 6 more for
+// the stored A_ij, where scaling every derivative took 65.  256^3: 1.97 -> 1.49
+// ms without the stores (48 operations at the measured FP64 rate: 1.52).
 template <bool STORE>
 __global__ void __launch_bounds__(kBlock)
     k_aij_aa(int lgn, double inv2h, double r, const double *__restrict__ Vx, const double *__restrict__ Vy,
@@ -213,15 +213,16 @@ __global__ void __launch_bounds__(kBlock)
             D[2][l] = V[l][io + jo + kp] - V[l][io + jo + km];
         }
         const double u0 = U[t];
-        const double S[3] = {U[ip + jo + k] + U[im + jo + k], U[io + jp + k] + U[io + jm + k],
-                             U[io + jo + kp] + U[io + jo + km]};
-        const double c = fma(-2.0 * r, u0, -0.5 * (D[0][0] + D[1][1] + D[2][2]));
+        // second differences of neighbouring values: nearly every subtraction is exact
+        const double S[3] = {fma(-2.0, u0, U[ip + jo + k]) + U[im + jo + k], fma(-2.0, u0, U[io + jp + k]) + U[io + jm + k],
+                             fma(-2.0, u0, U[io + jo + kp]) + U[io + jo + km]};
+        const double c = -0.5 * (D[0][0] + D[1][1] + D[2][2]);
         double Ad[3], Ao[3];
 #pragma unroll
         for (int a = 0; a < 3; a++) Ad[a] = fma(r, S[a], fma(2.0, D[a][a], c));
-        const double Xxy = (U[ip + jp + k] + U[im + jm + k]) - (U[im + jp + k] + U[ip + jm + k]);
-        const double Xxz = (U[ip + jo + kp] + U[im + jo + km]) - (U[im + jo + kp] + U[ip + jo + km]);
-        const double Xyz = (U[io + jp + kp] + U[io + jm + km]) - (U[io + jm + kp] + U[io + jp + km]);
+        const double Xxy = (U[ip + jp + k] - U[im + jp + k]) + (U[im + jm + k] - U[ip + jm + k]);
+        const double Xxz = (U[ip + jo + kp] - U[im + jo + kp]) + (U[im + jo + km] - U[ip + jo + km]);
+        const double Xyz = (U[io + jp + kp] - U[io + jm + kp]) + (U[io + jm + km] - U[io + jp + km]);
         Ao[0] = fma(r4, Xxy, D[0][1] + D[1][0]);
         Ao[1] = fma(r4, Xxz, D[0][2] + D[2][0]);
         Ao[2] = fma(r4, Xyz, D[1][2] + D[2][1]);
