@@ -52,7 +52,8 @@ BYTES = {
     "prolong32": {"any": 4.5},  # black children only (a red pass follows)
     "prolong64": {"any": 17.0},
     "mixed_resid": {"poisson": 20.0, "helm": 28.0, "psi": 44.0},
-    "df_resid": {"poisson": 22.0, "helm": 32.0, "psi": 46.0},  # + the first red pass of the next cycle
+    # helm, psi (and Poisson below 128^3, + 2): with the first red pass of the next cycle
+    "df_resid": {"poisson": 20.0, "helm": 32.0, "psi": 46.0},
     "mixed_update": {"any": 20.0},
     "df_black_update": {"poisson": 20.0, "helm": 22.0},  # last black pass + update of both colours
     "norm64": {"poisson": 16.0, "helm": 24.0, "psi": 32.0},
