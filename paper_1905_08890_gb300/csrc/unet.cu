@@ -122,13 +122,13 @@ void forward(gr_net *net, const gr_sources *s, double rho, double vrms)
     };
     cv(0);
     cv(1);
-    gr::pool(net->act[T_E0B], 16, 16, net->lg0, net->act[T_P1], st);
+    gr::pool(net->act[T_E0B], 16, net->lg0, net->act[T_P1], st);
     cv(2);
     cv(3);
-    gr::pool(net->act[T_E1B], 32, 32, net->lg0 - 1, net->act[T_P2], st);
+    gr::pool(net->act[T_E1B], 32, net->lg0 - 1, net->act[T_P2], st);
     cv(4);
     cv(5);
-    gr::pool(net->act[T_E2B], 64, 64, net->lg0 - 2, net->act[T_P3], st);
+    gr::pool(net->act[T_E2B], 64, net->lg0 - 2, net->act[T_P3], st);
     cv(6);
     cv(7);
     gr::upsample(net->act[T_E3B], 128, net->lg0 - 3, net->act[T_CAT2], 192, st);

@@ -30,7 +30,7 @@ int conv3d_tc_error(cudaStream_t st);
 // weight and bias gradients, added to dw and db
 void conv3d_wgrad(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *dy, int cout, int lg, float *dw, float *db,
                   cudaStream_t st);
-void pool(const __nv_bfloat16 *x, int c, int cstride, int lgf, __nv_bfloat16 *y, cudaStream_t st);
+void pool(const __nv_bfloat16 *x, int c, int lgf, __nv_bfloat16 *y, cudaStream_t st);
 void skip_back(const __nv_bfloat16 *dy, int c, int lgf, const __nv_bfloat16 *skip, int ss, int soff,
                const __nv_bfloat16 *act, __nv_bfloat16 *dx, cudaStream_t st);
 void upsample(const __nv_bfloat16 *x, int c, int lgc, __nv_bfloat16 *y, int cstride, cudaStream_t st);
