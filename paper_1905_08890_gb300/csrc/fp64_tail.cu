@@ -18,7 +18,7 @@
 // kind the black residuals, zero up to rounding, are not formed.
 // Measured at 32^3: the three levels and the 2^3 solve took 34 launches of 2
 // to 5 us each per linear cycle (psi: 240 us for the 2^3 sweeps alone); this
-// launch takes 27 us (74 us for psi).  With it, the finer prolongation and the
+// launch takes 27 us (69 us for psi).  With it, the finer prolongation and the
 // red-only restriction (mg_kernels.cu) a 32^3 FP64 solve of the ten equations
 // went from 19.1 to 8.8 ms.
 #include <cooperative_groups.h>
