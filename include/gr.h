@@ -167,7 +167,8 @@ typedef enum {
     GR_PROF_RESTRICT,      /* residual fused with restriction (FP64 or FP32) */
     GR_PROF_PROLONG,       /* trilinear prolongation + correction (FP64 or FP32) */
     GR_PROF_MIXED_RESID,   /* fine residual feeding the FP32 correction (mixed: FP64; mixed_df: double-float,
-                              with the correction's first red pass) */
+                              with the correction's first red pass, which Poisson grids from 128^3 leave to
+                              the black pass that follows) */
     GR_PROF_MIXED_UPDATE,  /* u += FP32 correction (mixed_df: fused with the last black pass) */
     GR_PROF_NORM64,        /* FP64 residual norm (FP64 path) */
     GR_PROF_SETUP,         /* sources, coefficients and layout changes of the finest level */
