@@ -31,8 +31,7 @@
 // 2.28 -> 1.94 ms.
 //
 // Blocks whose charges leave the scaled range (not finite, or 2^200 and more)
-// and particles at positions that are not finite or beyond 2^30 cells are added
-// directly in FP64.
+// and particles at positions that are not finite are added directly in FP64.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -57,17 +56,14 @@ struct Item {
 };
 
 // t = the argument times 2^shift: floor(t) and the fraction t - floor(t) in units of 2^-62 (positions below
-// 2^-62 of a cell are dropped), by integer operations on t's bits; far: t is
+// 2^-62 of a cell are dropped), by integer operations on t's bits; wide: t is
 // beyond 2^30 cells or not finite (no cell, no fraction)
-__device__ __forceinline__ int split_cell(double t, u64 &frac, bool &far, int shift = 0)
+__device__ __forceinline__ int split_cell(double t, u64 &frac, bool &wide, int shift = 0)
 {
     const long long b = __double_as_longlong(t);
     const int ex = (int)((b >> 52) & 0x7ff) - 1023 + shift;
-    if (ex >= 30) {
-        far = true;
-        frac = 0;
-        return 0;  // any cell: deposit_direct finds its own
-    }
+    wide = ex >= 30;
+    if (wide) return 0;
     const u64 m = ((u64)b & 0xfffffffffffffull) | 0x10000000000000ull;
     int c;
     u64 f;  // units of 2^-64
@@ -129,13 +125,35 @@ struct Grid {
     int lgh;  // invh = 2^lgh (exactly), or -1
 };
 
-// cell and fraction of coordinate x: t = x / h - 1/2.  With 1/h a power of two
-// (any box whose side is one) the scaling is an exponent and the half is
-// taken off the fraction: no FP64 operation.
-__device__ __forceinline__ int cell_of(const Grid &g, double x, u64 &frac, bool &far)
+// The FP64 form, for coordinates of 2^30 cells and more: wrapped into the grid as the
+// direct kernels wrap them.  bad: not finite, the fraction then is no number
+struct WideCell {
+    int lo;
+    bool bad;
+    u64 frac;
+};
+static __device__ __noinline__ WideCell cell_wide(double x, double invh, int m)
 {
-    if (g.lgh < 0) return split_cell(fma(x, g.invh, -0.5), frac, far);
-    int c = split_cell(x, frac, far, g.lgh);
+    const double t = fma(x, invh, -0.5), fl = floor(t), fr = t - fl;
+    const bool bad = !(fr < 1.0);
+    return {(int)((long long)fl & m), bad, bad ? 0ull : (u64)(fr * 0x1p62)};
+}
+
+// cell (to be wrapped into the grid) and fraction of coordinate x: t = x / h - 1/2.  With 1/h a power of two
+// (any box whose side is one) the scaling is an exponent and the half is
+// taken off the fraction: no FP64 operation.  Both passes call it, so a particle is summed in the tile it
+// was counted in.
+__device__ __forceinline__ int cell_of(const Grid &g, double x, u64 &frac, bool &bad)
+{
+    bool wide;
+    int c = split_cell(g.lgh < 0 ? fma(x, g.invh, -0.5) : x, frac, wide, g.lgh < 0 ? 0 : g.lgh);
+    if (wide) {
+        const WideCell w = cell_wide(x, g.invh, (1 << g.lgn) - 1);
+        frac = w.frac;
+        bad |= w.bad;
+        return w.lo;
+    }
+    if (g.lgh < 0) return c;
     const u64 half = 1ull << 61;
     if (frac < half) c--;
     frac = (frac - half) & ((1ull << 62) - 1);
@@ -162,8 +180,8 @@ __global__ void __launch_bounds__(kBlock)
 #pragma unroll
         for (int d = 0; d < 3; d++) {
             u64 f;
-            bool far;
-            lo[d] = cell_of(g, x[d * stride + p], f, far);
+            bool bad = false;
+            lo[d] = cell_of(g, x[d * stride + p], f, bad);
         }
     }
     const unsigned tile = ok ? tile_of(g, lo) : 0xffffffffu;
@@ -272,20 +290,23 @@ __device__ __forceinline__ double rsqrt64(double a)
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
-// one particle straight to memory in FP64
-static __device__ __noinline__ void deposit_direct(const Grid g, double q, double x, double y, double z, double ux,
-                                                   double uy, double uz, const double *psi, const Out out)
+// One particle straight to memory in FP64.  (cx, cy, cz), f: its cell and fractions by cell_of, so that it
+// adds to no cells but those its tile reaches (cells inside another tile may take that tile's plain
+// stores at any time); a coordinate that is not finite has no fraction and spoils its cells.
+static __device__ __noinline__ void deposit_direct(const Grid g, double q, double x, double y, double z, int cx, int cy,
+                                                   int cz, u64 f0, u64 f1, u64 f2, double ux, double uy, double uz,
+                                                   const double *psi, const Out out)
 {
     const int m = (1 << g.lgn) - 1;
     const double x3[3] = {x, y, z};
-    int lo[3];
+    const u64 f[3] = {f0, f1, f2};
+    const int lo[3] = {cx, cy, cz};
     double fw[3][2];
 #pragma unroll
     for (int d = 0; d < 3; d++) {
-        const double t = fma(x3[d], g.invh, -0.5), fl = floor(t), fr = t - fl;
+        const double t = x3[d] * g.invh, fr = (double)f[d] * 0x1p-62 + (t - t);  // + 0, or NaN
         fw[d][0] = 1.0 - fr;
         fw[d][1] = fr;
-        lo[d] = (int)((long long)fl & m);
     }
     auto id = [&](int a, int b, int c) {
         return (((((lo[0] + a) & m) << g.lgn) + ((lo[1] + b) & m)) << g.lgn) + ((lo[2] + c) & m);
@@ -389,15 +410,16 @@ __global__ void __launch_bounds__(kSegThreads, 5)
         int lc[3];
         u64 f[3];
         double fr[3];
-        bool far = false;
+        bool bad = false;
 #pragma unroll
         for (int d = 0; d < 3; d++) {
-            lc[d] = cell_of(g, xd[d], f[d], far) & (kTile - 1);
+            lc[d] = cell_of(g, xd[d], f[d], bad) & (kTile - 1);
             if (METRIC) fr[d] = f[d] ? from_units((long long)f[d], -62) : 0.0;
         }
-        if (!scaled || far) {
+        if (!scaled || bad) {
             direct = 1u;
-            deposit_direct(g, q, xd[0], xd[1], xd[2], ud[0], ud[1], ud[2], METRIC ? psi : nullptr, out);
+            deposit_direct(g, q, xd[0], xd[1], xd[2], base[0] + lc[0], base[1] + lc[1], base[2] + lc[2], f[0], f[1], f[2],
+                           ud[0], ud[1], ud[2], METRIC ? psi : nullptr, out);
             continue;
         }
         const int r0 = (lc[0] * kReach + lc[1]) * kReach + lc[2];
