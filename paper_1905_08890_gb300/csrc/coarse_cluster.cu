@@ -374,12 +374,12 @@ cudaLaunchConfig_t cluster_config(cudaStream_t st, cudaLaunchAttribute *at)
     return cfg;
 }
 
-// once per kind: the 16-CTA cluster (beyond the portable 8) and its shared
+// once per kind and device: the 16-CTA cluster (beyond the portable 8) and its shared
 // memory are allowed, and the device can hold one such cluster
 template <int KIND>
 bool cluster_usable()
 {
-    static const bool ok = [] {
+    return per_device([] {
         auto k = k_coarse_cluster<KIND>;
         if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmem) != cudaSuccess) {
@@ -395,8 +395,7 @@ bool cluster_usable()
             return false;
         }
         return nc >= 1;
-    }();
-    return ok;
+    });
 }
 
 template <int KIND>

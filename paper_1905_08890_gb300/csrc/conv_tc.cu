@@ -403,9 +403,12 @@ void launch_tc(const __nv_bfloat16 *x, const __nv_bfloat16 *w, const float *bias
         int dev = 0, n = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(k_conv3d_tc<NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Ring<NCH>::kSmem);
         return n > 0 ? n : 1;
     }();
+    per_device([] {
+        return cudaFuncSetAttribute(k_conv3d_tc<NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)Ring<NCH>::kSmem) == cudaSuccess;
+    });
     // one block per SM (its tensor memory) and group of 16 output channels
     const dim3 grid(sms < kUnits ? sms : kUnits, cout / 16);
     GR_LAUNCH_SMEM((k_conv3d_tc<NCH>), grid, kThreads, (int)Ring<NCH>::kSmem, st, x, w, bias, cout, mode, mask, y);

@@ -355,11 +355,11 @@ cudaLaunchConfig_t tail64_config(cudaStream_t st, cudaLaunchAttribute *at)
     return cfg;
 }
 
-// once per kind: the 16-CTA cluster (beyond the portable 8) is allowed and fits the device
+// once per kind and device: the 16-CTA cluster (beyond the portable 8) is allowed and fits the device
 template <int KIND>
 bool tail64_usable()
 {
-    static const bool ok = [] {
+    return per_device([] {
         auto k = k_tail64<KIND>;
         cudaLaunchAttribute at[2];
         cudaLaunchConfig_t cfg = tail64_config<KIND>(nullptr, at);
@@ -371,8 +371,7 @@ bool tail64_usable()
             return false;
         }
         return nc >= 1;
-    }();
-    return ok;
+    });
 }
 
 template <int KIND>

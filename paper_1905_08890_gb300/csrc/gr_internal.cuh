@@ -20,6 +20,7 @@
 #include <mutex>
 #include <unordered_map>
 
+#include "device_once.cuh"
 #include "df64.cuh"
 
 namespace gr {
@@ -69,6 +70,17 @@ inline void launch_pdl(void (*k)(KArgs...), dim3 g, dim3 b, size_t smem, cudaStr
         ::gr::launch_pdl(kernel, (grid), (block), (smem), (stream), __VA_ARGS__); \
         ::gr::g_launches.fetch_add(1, std::memory_order_relaxed);                \
     } while (0)
+
+// f() once for each device it is called on (a kernel's attributes, such as its dynamic shared
+// memory, belong to one device), its result on every call.  One set-up per type F: call it with a lambda.
+template <class F>
+bool per_device(F &&f)
+{
+    static DeviceOnce once;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return once(dev, f);
+}
 
 #ifdef __CUDACC__
 // first statement of every kernel: let the stream's next kernel launch, then

@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(C::T)
     }
 }
 
-// the shared-memory opt-in, once per kernel.  The carve-out is held to one
+// the shared-memory opt-in, once per kernel and device.  The carve-out is held to one
 // block per SM: left to itself the driver makes room for as many blocks as the
 // SM could take, and the kernels that follow (which state no preference) then
 // run with what L1 is left, 10% slower over a 512^3 solve.
@@ -344,8 +344,7 @@ template <class C, int KIND, bool FROM_R>
 void down_t(const float *e, float *eb, const float *r, const float *m, const float *inv, double h2, double ih2, float *ec,
             float *rc, const float *cinv, double h2c, cudaStream_t st)
 {
-    static const bool attr = opt_in<C>(k_level_down<C, KIND, FROM_R>);
-    (void)attr;
+    per_device([] { return opt_in<C>(k_level_down<C, KIND, FROM_R>); });
     GR_LAUNCH_SMEM((k_level_down<C, KIND, FROM_R>), C::BLOCKS, C::T, C::SMEM, st, e, eb, r, m, inv, (float)h2, (float)ih2,
                    ec, rc, cinv, (float)h2c);
 }
@@ -354,8 +353,7 @@ template <class C, int KIND, bool UPDATE>
 void up_t(float *e, const float *eb, const float *r, const float *inv, const float *ec, double h2, float *uh, float *ul,
           cudaStream_t st)
 {
-    static const bool attr = opt_in<C>(k_level_up<C, KIND, UPDATE>);
-    (void)attr;
+    per_device([] { return opt_in<C>(k_level_up<C, KIND, UPDATE>); });
     GR_LAUNCH_SMEM((k_level_up<C, KIND, UPDATE>), C::BLOCKS, C::T, C::SMEM, st, e, eb, r, inv, ec, (float)h2, uh, ul);
 }
 

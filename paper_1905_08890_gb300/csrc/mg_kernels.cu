@@ -1108,17 +1108,18 @@ void coarse_tail(int kind, float *const *e, float *const *r, const float *const 
         a.inv[l] = inv[l];
         a.h2[l] = (float)h2[l];
     }
-    const size_t smem = sizeof(float) * 4 * (8 + 64 + 512 + 4096);  // e, r, m, inv
-    // once per kernel (function-local statics are initialised once, even with several host threads)
+    constexpr int smem = (int)sizeof(float) * 4 * (8 + 64 + 512 + 4096);  // e, r, m, inv
     if (kind == KPOISSON) {
-        static const bool attr = cudaFuncSetAttribute(k_coarse_tail<KPOISSON>,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
-        (void)attr;
+        per_device([] {
+            return cudaFuncSetAttribute(k_coarse_tail<KPOISSON>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
+                   cudaSuccess;
+        });
         GR_LAUNCH_SMEM(k_coarse_tail<KPOISSON>, 1, kTailThreads, smem, st, a, nu1, nu2);
     } else {
-        static const bool attr = cudaFuncSetAttribute(k_coarse_tail<KHELM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)smem) == cudaSuccess;
-        (void)attr;
+        per_device([] {
+            return cudaFuncSetAttribute(k_coarse_tail<KHELM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) ==
+                   cudaSuccess;
+        });
         GR_LAUNCH_SMEM(k_coarse_tail<KHELM>, 1, kTailThreads, smem, st, a, nu1, nu2);
     }
 }

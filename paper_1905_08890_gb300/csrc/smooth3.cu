@@ -374,10 +374,10 @@ void launch_s3(void (*kern)(S3Args), int n, const float *ein, float *eout, const
 {
     const S3Layout<KIND, D> L{kTJMax};
     const size_t smem = (size_t)L.total() * sizeof(float4);
-    // once per kernel (a function-local static is initialised once, even with several host threads)
-    static const bool attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-                             cudaSuccess;
-    (void)attr;
+    // KIND and D name the kernel
+    per_device([&] {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+    });
     int lgn = 0;
     while ((1 << lgn) < n) ++lgn;
     S3Args a{ein, eout, f, g, (float)h2, lgn, c1, rt};

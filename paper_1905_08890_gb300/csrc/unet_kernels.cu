@@ -236,9 +236,10 @@ void launch_conv3d(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, cons
 {
     // the largest halo of these boxes: 2^8 voxels as 4 x 4 x 16 or 4 x 8 x 8
     constexpr int kMost = 2 * 32 * (720 + 27 * NT * 8);
-    static const bool attr = cudaFuncSetAttribute(k_conv3d<WARPS, MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  kMost) == cudaSuccess;
-    (void)attr;
+    per_device([] {
+        return cudaFuncSetAttribute(k_conv3d<WARPS, MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) ==
+               cudaSuccess;
+    });
     const Box bx = make_box(lg, lb);
     const int smem = (cin > 16 ? 2 : 1) * 32 * (bx.halo() + 27 * NT * 8);
     const dim3 grid(1u << (3 * lg - lb), cout / (NT * 8));
@@ -895,9 +896,9 @@ void conv3d_wgrad(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *dy, int 
     int split = (4 * 152 + pairs - 1) / pairs;
     if (split > nbox) split = nbox;
     constexpr int kMost = 2 * 32 * (720 + (1 << kWgBox));
-    static const bool attr =
-        cudaFuncSetAttribute(k_conv3d_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) == cudaSuccess;
-    (void)attr;
+    per_device([] {
+        return cudaFuncSetAttribute(k_conv3d_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost) == cudaSuccess;
+    });
     const int smem = 2 * 32 * (bx.halo() + (1 << lb));
     GR_LAUNCH_SMEM(k_conv3d_wgrad, dim3(split, pairs), 32 * kWgWarps, smem, st, x, cin, dy, cout, bx, nbox, dw, db);
 }
