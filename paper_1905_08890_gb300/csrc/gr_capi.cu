@@ -100,7 +100,9 @@ struct gr_ctx {
     // the psi, alpha psi in the fields: 0 nothing current, 1 FP64, 2 double-float pairs, 3 AA in FP64 alone
     int a_fmt = 0;
     int w_fmt = 0;
-    bool tail_on = true;   // FP32 cycles: levels <= 16^3 in one block (GR_COARSE_TAIL=0 turns it off)
+    // GR_COARSE_TAIL=0 turns it off: FP32 cycles' levels <= 16^3 in one block and 32^3, 64^3 in one launch per
+    // direction, FP64 cycles' levels <= 16^3 in one cluster, the full multigrid start
+    bool tail_on = true;
     bool cluster_on = false;  // FP32 cycles under a 128^3 or finer top: levels <= 64^3 in one
                               // 16-CTA cluster (GR_COARSE_CLUSTER=1; measured slower)
     int s3_min = 1 << 30;  // finest grids from this size fuse three colour passes per smoothing: off unless
@@ -1159,11 +1161,13 @@ long long patch_cells(const gr_ctx *c, int nu)
 }
 
 // Solve (or cycle) one equation; writes the field back.  tol < 0 with
-// max_cycles = 1 performs exactly one cycle and reports OK.
+// max_cycles = 1 performs exactly one cycle and reports OK.  may_queue: a cycle
+// may be queued before its predecessor's norm is known.
 gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const gr_opts *o, double rho,
                    double S_hat, double tol, int max_cycles, int *cycles, double *res0, double *res,
-                   long long *cells, int *rejected = nullptr, double *res_level = nullptr)
+                   long long *cells, int *rejected = nullptr, double *res_level = nullptr, bool may_queue = true)
 {
+    const long long cells0 = cells ? *cells : 0;
     EqInfo in;
     gr_status st = GR_OK;
     const bool dfm = o->prec == GR_PREC_MIXED_DF;
@@ -1260,9 +1264,12 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
     int cyc = 0;
     if (!std::isfinite(r)) st = fail(GR_ERR_NONFINITE, "equation %d: initial residual is not finite", eq);
     // While the residual is more than 1e4 above the tolerance the cycle after the
-    // next is certain to run (a V-cycle gains a factor of ten): it is queued
-    // without waiting for the next one's norm, which is read while it runs.
-    const bool ahead = !patches && !check && !c->prof_on;
+    // next hardly ever turns out superfluous (a V-cycle gains a factor of ten, more only
+    // on special right-hand sides or with many sweeps): it is queued without waiting for the
+    // next one's norm, which is read while it runs.  If that norm ends the solve after all, the
+    // fields have gone one cycle too far, and the equation is solved again from the guess, which
+    // is still in fl, without queueing: the result is then that of reading every norm first.
+    const bool ahead = may_queue && !patches && !check && !c->prof_on;
     bool unread = false;  // a norm is queued whose value r does not hold yet
     auto finite = [&] {
         if (st == GR_OK && !std::isfinite(r)) st = fail(GR_ERR_NONFINITE, "equation %d: residual not finite", eq);
@@ -1300,7 +1307,11 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
             queue_norm();
             if (unread) {
                 st = read_norm(c, dfm ? 1.0 : in.ref, &r, 1);
-                finite();
+                if (st == GR_OK && !(std::isfinite(r) && r > tol)) {
+                    if (cells) *cells = cells0;
+                    return solve_eq(c, eq, s, fl, o, rho, S_hat, tol, max_cycles, cycles, res0, res, cells, rejected,
+                                    res_level, false);
+                }
             }
             unread = st == GR_OK && r > 1e4 * tol && cyc < max_cycles;
             if (!unread && st == GR_OK) st = read_norm(c, dfm ? 1.0 : in.ref, &r);
