@@ -83,11 +83,21 @@ bool per_device(F &&f)
 }
 
 #ifdef __CUDACC__
-// first statement of every kernel: let the stream's next kernel launch, then
-// wait for the previous one (a no-op for a kernel launched without the attribute)
+// First statement of every kernel: let the stream's next kernel launch, then
+// wait for the previous one (a no-op for a kernel launched without the attribute).
+// The wait alone does not hold back every load that follows it: what a kernel reads
+// through const __restrict__ pointers or __ldg counts as constant while it runs, and the
+// compiler moved such loads above the wait (a list's length was read before the kernel that
+// writes it had ended).  A load may not be moved above a branch that decides whether it is made,
+// so a branch the compiler cannot decide follows the wait: no SM has the number 2^32 - 1.
 __device__ __forceinline__ void pdl_begin()
 {
-    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+    unsigned sm;
+    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;\n\tmov.u32 %0, %%smid;" : "=r"(sm)::"memory");
+    if (sm == 0xffffffffu) {
+        asm volatile("exit;");
+        __builtin_unreachable();
+    }
 }
 #endif
 
