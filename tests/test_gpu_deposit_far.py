@@ -13,11 +13,10 @@ if not torch.cuda.is_available():  # pragma: no cover - the gpu marker deselects
 
 from paper_1905_08890_gb300 import gr  # noqa: E402
 
-N = 128
 MASS = 1e-7
 
 
-def _set(L, seed, npart=N ** 3):
+def _set(N, L, seed, npart):
     """npart particles at speeds of 0.3 (enough of them for the tiles), and the inner cells of tiles, all over the
     box, for 4000 more."""
     g = torch.Generator(device="cuda").manual_seed(seed)
@@ -29,7 +28,7 @@ def _set(L, seed, npart=N ** 3):
 
 def _deposit(ctx, x, u, metric):
     if metric:
-        psi = torch.full((N, N, N), 1.1, dtype=torch.float64, device="cuda")
+        psi = torch.full((ctx.n,) * 3, 1.1, dtype=torch.float64, device="cuda")
         src = ctx.deposit_metric(x.contiguous(), u.contiguous(), MASS, psi)
     else:
         src = ctx.deposit(x.contiguous(), u.contiguous(), MASS)
@@ -47,7 +46,8 @@ def test_far_positions_are_wrapped(axis, sign, L, metric):
     rounded position is wrapped in exact integer arithmetic for the comparison."""
     from fractions import Fraction
 
-    x, cell, u = _set(L, 11 + axis, (2 if metric else 1) * N ** 3)
+    N = 256 if metric else 128  # the sets that the tiles take
+    x, cell, u = _set(N, L, 11 + axis, (3 if metric else 2) * N ** 3 // 2)
     h = L / N
     near = (cell.to(torch.float64) + 0.75) * h
     far = near.clone()
@@ -71,7 +71,8 @@ def test_far_positions_are_wrapped(axis, sign, L, metric):
 def test_extreme_positions_are_those_of_the_direct_kernel(L):
     """Up to 1e300, infinite and NaN: the tiled deposit equals its finite part plus each such particle on its own
     (one particle takes the direct kernel), including which cells become NaN."""
-    x, _, u = _set(L, 21)
+    N = 128
+    x, _, u = _set(N, L, 21, N ** 3)
     u = u[:, : x.shape[1]]
     h = L / N
     inf, nan = float("inf"), float("nan")
