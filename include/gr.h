@@ -185,8 +185,8 @@ typedef struct {
     gr_status eq_status[GR_NEQ];
     double seconds;               /* wall time of the whole call (host clock around the stream) */
     double eq_seconds[GR_NEQ];    /* per equation, CUDA events */
-    long long cell_updates;       /* cells relaxed: every sweep on every level, all equations (the exact
-                                     solve of a linear 2^3 level counts its 8 cells once) */
+    long long cell_updates;       /* cells relaxed: every sweep on every level, all equations (the 2^3 level's 8
+                                     cells count once per cycle, solved exactly or by Newton's method) */
     long long kernel_launches;    /* kernels this call launched */
     int prof_launches[GR_NPROF];  /* with gr_opts.profile: launches per gr_prof_class */
     double prof_ms[GR_NPROF];     /* with gr_opts.profile: summed CUDA-event time per class */

@@ -484,7 +484,8 @@ void restrict_coefs32(gr_ctx *c)
 
 // cells relaxed by one V-cycle whose top is level top (default: the finest);
 // coarsest: the cell updates of the 2^3 solve (8 for the exact solve of a
-// linear level, 8 per sweep for the nonlinear one)
+// linear level and for Newton's method on the nonlinear one, which the cluster launch
+// takes; 8 per sweep for that level's separate launch)
 long long vcycle_cells(const gr_ctx *c, int nu1, int nu2, int top = -1, long long coarsest = 8)
 {
     if (top < 0) top = c->nlev - 1;
@@ -500,6 +501,9 @@ long long fmg_cells(const gr_ctx *c, int nu1, int nu2)
     for (int l = 4; l < c->nlev; l++) s += vcycle_cells(c, nu1, nu2, l);
     return s;
 }
+
+// whether an FP64 cycle's levels up to 16^3 run in one launch
+bool uses_tail64(const gr_ctx *c, int kind) { return c->tail_on && gr::tail64_ok(kind); }
 
 // Relaxation and transfers of one V-cycle.  With profiling, the finest
 // level's launches are timed per class and everything below it (which runs
@@ -528,7 +532,7 @@ void vcycle64(gr_ctx *c, int kind, double rho, int nu1, int nu2)
         gr::prolong_add64(A.n, A.u, C.u, !fas && nu2 > 0, c->st);
     };
     // levels up to 16^3 run in one launch
-    const int low = (c->tail_on && gr::tail64_ok(kind)) ? std::min(top, 3) : 0;
+    const int low = uses_tail64(c, kind) ? std::min(top, 3) : 0;
     auto coarse = [&] {
         for (int l = top - 1; l > low; l--) {
             smooth(c->lev[l], nu1);
@@ -1212,8 +1216,8 @@ gr_status solve_eq(gr_ctx *c, int eq, const gr_sources *s, gr_fields *fl, const 
         }
     }
     const bool mixed = o->prec == GR_PREC_MIXED || dfm;
-    const long long per_cycle =
-        vcycle_cells(c, o->nu1, o->nu2, -1, (!mixed && in.kind == KPSI) ? 8LL * kCoarsestSweeps : 8LL);
+    const bool swept = !mixed && in.kind == KPSI && !uses_tail64(c, in.kind);  // the 2^3 level
+    const long long per_cycle = vcycle_cells(c, o->nu1, o->nu2, -1, swept ? 8LL * kCoarsestSweeps : 8LL);
     if (mixed) {
         if (in.kind == KHELM) {
             if (!dfm) {  // the double-float set-up wrote m and its inverse diagonal
