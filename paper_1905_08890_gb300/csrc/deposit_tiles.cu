@@ -314,20 +314,6 @@ struct Out {
     double *s[5];
 };
 
-// 1/sqrt(a), a >= 1: the FP32 estimate and one third-order step
-// y <- y (1 + e/2 + 3 e^2/8), e = 1 - a y^2 (the binomial series of (1 - e)^-1/2)
-__device__ __forceinline__ double rsqrt64(double a)
-{
-    if (!(a < 0x1p120)) return rsqrt(a);
-    // a's leading 24 bits as a float and y back, by moving exponent and mantissa
-    const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a);
-    const float f = __uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29));
-    const unsigned yb = __float_as_uint(rsqrtf(f));
-    const double y = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
-    const double e = fma(-a * y, y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
-
 // One particle straight to memory in FP64.  (cx, cy, cz), f: its cell and fractions by cell_of, so that it
 // adds to no cells but those its tile reaches (cells inside another tile may take that tile's plain
 // stores at any time); a coordinate that is not finite has no fraction and spoils its cells.

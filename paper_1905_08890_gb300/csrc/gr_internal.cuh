@@ -175,14 +175,34 @@ struct Sums {
 // the first red relaxation of a Poisson correction from e = 0 (rounded as if stored: not contracted into the sum it enters)
 __device__ __forceinline__ float first_red(float r, float h2) { return __fmul_rn(__fmul_rn(-h2, r), 1.0f / 6.0f); }
 
+// The divisions for recip64's rare operands, out of line so that they do not occupy the common path
+static __device__ __noinline__ double recip64_any(double x) { return 1.0 / x; }
+
 // 1/x by Newton's iteration r <- r + r (1 - x r) from the hardware's 20-bit
-// estimate: two steps leave about one unit in the last place
+// estimate: two steps leave at most one unit in the last place.  The iteration has no zeros, infinities
+// and subnormals (of x or of the result): those x are divided
 __device__ __forceinline__ double recip64(double x)
 {
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+    if (ex - 1u > 2043u) return recip64_any(x);
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     r = fma(r, fma(-x, r, 1.0), r);
     return fma(r, fma(-x, r, 1.0), r);
+}
+
+// 1/sqrt(a), a >= 1: the FP32 estimate and one third-order step
+// y <- y (1 + e/2 + 3 e^2/8), e = 1 - a y^2 (the binomial series of (1 - e)^-1/2): at most two units in the last place
+__device__ __forceinline__ double rsqrt64(double a)
+{
+    if (!(a < 0x1p120)) return rsqrt(a);
+    // a's leading 24 bits as a float and y back, by moving exponent and mantissa
+    const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a);
+    const float f = __uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29));
+    const unsigned yb = __float_as_uint(rsqrtf(f));
+    const double y = __hiloint2double((int)((yb >> 3) + (896u << 20)), (int)(yb << 29));
+    const double e = fma(-a * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 // Sums of a and b over the warp's lanes: lane 0 returns a's, lane 16 b's.  The lower half goes on with a
