@@ -51,7 +51,7 @@ struct T64Smem {
     double part[2 * 340], partu[2 * 340];  // 8-child sums from the two fine planes
     double cb[2 * 340];  // coarser level's correction for this CTA's plane: own and neighbouring coarse plane
     double zf[2][2][4], zu[2][2][4];       // the 2^3 level's incoming sums [plane][half][cell]
-    double zs[8], z0[8], z1[8], zr[8], zb[8];
+    double z0[8], z1[8], zb[8];
 };
 
 // N(u) at a cell without its right-hand side; nb the neighbour sum
@@ -190,8 +190,7 @@ struct Tail64 {
     // trilinear prolongation onto level l (3/4 and 1/4 per axis)
     __device__ void up(int l, bool black_only)
     {
-        const int n = 2 << l, nc = n / 2, mc = nc - 1, po = plane_off(l), pc = plane_off(l - 1);
-        (void)po;
+        const int n = 2 << l, nc = n / 2, mc = nc - 1, pc = plane_off(l - 1);
         if (l > 1) {
             if (r < nc)
                 for (int t = threadIdx.x; t < nc * nc; t += kT64Threads)

@@ -29,20 +29,9 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__device__ __forceinline__ uint32_t ld32(const __nv_bfloat16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
-
 __device__ __forceinline__ uint32_t pack2(__nv_bfloat16 lo, __nv_bfloat16 hi)
 {
     return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
-
-// neighbour voxel of v at tap (wrapped, grid 2^lg per axis)
-__device__ __forceinline__ int nbr(int v, int lg, int tap)
-{
-    const int m = (1 << lg) - 1;
-    const int w = v & m, h = (v >> lg) & m, d = v >> (2 * lg);
-    const int dd = tap / 9 - 1, dh = (tap / 3) % 3 - 1, dw = tap % 3 - 1;
-    return ((((d + dd) & m) << lg) + ((h + dh) & m)) * (1 << lg) + ((w + dw) & m);
 }
 
 // ---------------------------------------------------------------- convolution
@@ -247,7 +236,7 @@ void launch_conv3d(const __nv_bfloat16 *x, int cin, const __nv_bfloat16 *w, cons
 }
 
 // ---------------------------------------------------------------- weight gradient
-// dw[tap][co][ci] += sum_v dy[v][co] x[nbr(v, tap)][ci]: GEMM with M = co,
+// dw[tap][co][ci] += sum_v dy[v][co] x[v's neighbour at tap][ci]: GEMM with M = co,
 // N = ci, K = voxels.  Block: 16 output x 16 input channels (grid.y), a range of
 // voxel boxes (grid.x), all 27 taps, three per warp.  Per box the 16 channels of
 // dy and of x with its halo are staged in shared memory, one box ahead; both
