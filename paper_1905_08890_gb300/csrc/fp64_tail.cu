@@ -247,10 +247,12 @@ struct Tail64 {
                 const double m = fma(2.0 * kPi * c0, iv2, (0.875 * c1) * (iv4 * iv4)) + (10.0 * kPi * A.rho) * v4;
                 const double d = coarsest_exact<KHELM>(f - op64<KPSI>(nb(u), u, c0, c1, ih2, A.rho), m, h2);
                 u += d;
+                // a step out of the positive conformal factors may end at a root beyond the pole at zero
+                if (__any_sync(full, __double2hiint(1.0 + u) <= 0)) break;
                 // the next step would move u by less than its rounding
                 done = __all_sync(full, d * d <= 0x1p-56 * fabs(u) || d == 0.0);
             }
-            if (!done) {  // far from the solution: red-black Newton sweeps and the zero-mode shift, as k_coarsest
+            if (!done) {  // far from the solution (one in a thousand of random strong defects): red-black Newton sweeps and the zero-mode shift, as k_coarsest
                 const int color = __popc(x) & 1;
                 u = ur;
                 for (int sweep = 0; sweep < kCoarsestSweeps; sweep++) {
