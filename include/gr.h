@@ -224,7 +224,9 @@ void gr_destroy(gr_ctx *ctx);
    A mix of host and device pointers is GR_ERR_ARG.  Each particle adds, with CIC
    weight w over the 8 surrounding cell centres, m W w/h^3 to s0,
    m u_l w/h^3 to s_l and m |u|^2/W w/h^3 to sigma, W = sqrt(1 + |u|^2)
-   (the conformal factor is taken as 1 in the Lorentz factor).  The five
+   (the conformal factor is taken as 1 in the Lorentz factor).  A cell's sums are
+   good to about 2^-46 of the sum of its charges' magnitudes, whatever the others are;
+   charges meet in FP64 atomics, so their last bits can differ between calls.  The five
    output arrays are overwritten.  np = 0 gives zero sources.  Also records
    mass*np/L^3 as the default rho_hat of the context. */
 gr_status gr_deposit(gr_ctx *ctx, int64_t np, const double *x, const double *u, double mass, gr_sources *out);

@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kBlock)
 // records of 64 cells at a time (5120 contiguous bytes) go through shared memory so
 // that the stores are consecutive (a slot in forty is skipped, which spreads the
 // lanes over the banks).  32-bit offsets: n <= 1024.  Memory bound: 100 bytes per
-// cell, 2.4 ms at 512^3 (6.9 with one cell per thread and 35 scalar loads).
+// cell, 3.2 ms at 512^3 (6.9 with one cell per thread and 35 scalar loads).
 __global__ void __launch_bounds__(kBlock)
     k_pf_grad(int lgn, float inv2h, const float *__restrict__ d, float4 *__restrict__ rec)
 {
@@ -289,7 +289,7 @@ __device__ __forceinline__ Cloud cloud(double x, double invh, int lgh)
 // quadruple v of the records around particle s of six, with that particle's cells and
 // weights from shared memory, and leaves the interpolated quadruple there.
 // top: below L by a relative 2^-40.  Latency and L1 bound (L1 75% busy, records of
-// scattered particles; 4 blocks of 64 registers, 5 spill): 12.6 -> 10.2 ms for
+// scattered particles; 4 blocks of 64 registers, 5 spill): 12.6 -> 10.4 ms for
 // 134M particles.
 __global__ void __launch_bounds__(kBlock, 4)
     k_particle_update(int lgn, double invh, int lgh, double L, double invL, double top, int64_t np,
