@@ -32,8 +32,8 @@
 //
 // Bound: integer multiplies and the additions' bank conflicts (four wavefronts each for clustered
 // particles), at 62% occupancy (48 registers; 4 blocks of 60 registers took 4%
-// more).  Measured, 134M particles on 512^3, rms contrast 5: 18.8 -> 15.0 ms
-// (order 2.0 ms, sums 11.6 ms, list 0.7 ms, zeroing 0.8 ms; without the list and the bounds per cell 12.8).
+// more).  Measured, 134M particles on 512^3, rms contrast 5: 18.8 -> 15.2 ms
+// (order 2.0 ms, sums 11.8 ms, list 0.7 ms, zeroing 0.8 ms; without the list and the bounds per cell 12.8).
 //
 // Items whose charges leave the scaled range (not finite, or 2^200 and more)
 // and particles at positions that are not finite are listed with all their charges.
@@ -546,8 +546,9 @@ __global__ void __launch_bounds__(kSegThreads, 5)
 #pragma unroll
                 for (int c = 0; c < 2; c++) {
                     const int r = r0 + (a * kReach + b) * kReach + c;
-                    const int sc = scale[r];
-                    const u64 wt = mul62(wab, w[2][c]) >> (sc & 7);
+                    const int sc = scale[r], drop = sc & 7;
+                    // rounded: a crowd's truncations would add up (twice the error at 3e-4 of a cell's side from its edge)
+                    const u64 wt = (mul62(wab, w[2][c]) + ((1u << drop) >> 1)) >> drop;
                     const int wh = (int)(wt >> 31), wl = (int)(wt & 0x7fffffffull);
 #pragma unroll
                     for (int k = 0; k < 5; k++) {
