@@ -32,8 +32,8 @@
 //
 // Bound: integer multiplies and the additions' bank conflicts (four wavefronts each for clustered
 // particles), at 62% occupancy (48 registers; 4 blocks of 60 registers took 4%
-// more).  Measured, 134M particles on 512^3, rms contrast 5: 18.8 -> 15.2 ms
-// (order 2.0 ms, sums 11.8 ms, list 0.7 ms, zeroing 0.8 ms; without the list and the bounds per cell 12.8).
+// more).  Measured, 134M particles on 512^3, rms contrast 5: 18.8 -> 15.4 ms
+// (order 2.2 ms, sums 11.8 ms, list 0.7 ms, zeroing 0.8 ms; without the list and the bounds per cell 12.8).
 //
 // Items whose charges leave the scaled range (not finite, or 2^200 and more)
 // and particles at positions that are not finite are listed with all their charges.
